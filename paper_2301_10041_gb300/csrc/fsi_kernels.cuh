@@ -56,7 +56,6 @@ struct Ctl {
   int refine;       // 1 when the current Gram-Schmidt step needs a second pass
   int max_cycles;   // cap on restart / refinement cycles of one solve
   int refines;      // second passes taken in this solve
-  double wnorm2;    // ||w||^2 before orthogonalisation
   unsigned int counter[8];  // last-block counters for reductions
 };
 
@@ -335,6 +334,8 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 16 : 8) k_resrestrict(Se
 // y = alpha * A x + beta * z for the block operator of Eq. (matrix) in the
 // layout [u (2 nU) | p (3 nP) | X (2 nS) | lambda (2 nS)].  One launch covers
 // the three row segments; each CTA (4 warps, 32 block rows) lies in one.
+// With Z given, x is also stored as its column ctl->j (the flexible GMRES
+// direction), each CTA copying its own rows.
 template <class TA>
 struct FullOp {
   int nU = 0, nP = 0, nS = 0;
@@ -353,12 +354,28 @@ struct FullOp {
 
 template <class TA, class TX, class TY>
 __global__ void __launch_bounds__(128, sizeof(TA) == 4 ? 16 : 8) k_fullmv(FullOp<TA> op, const TX* __restrict__ x, TY* __restrict__ y,
-                                                const TY* __restrict__ z, TY alpha, TY beta) {
+                                                const TY* __restrict__ z, TY alpha, TY beta,
+                                                TX* __restrict__ Z, size_t zld, const Ctl* __restrict__ ctl) {
   pdl_begin();
   const int lane = threadIdx.x & 31, t = lane >> 3;
   const int b = blockIdx.x;
   const int wrow = (threadIdx.x >> 5) * kSliceRows + (lane & 7);
   const size_t offP = 2 * (size_t)op.nU, offX = offP + 3 * (size_t)op.nP, offL = offX + 2 * (size_t)op.nS;
+  if (Z) {
+    TX* Zc = Z + (size_t)ctl->j * zld;
+    const int i = threadIdx.x;
+    if (b < op.gU) {
+      const int c = 64 * b + i;
+      if (i < 64 && c < 2 * op.nU) Zc[c] = x[c];
+    } else if (b < op.gU + op.gP) {
+      const int c = 96 * (b - op.gU) + i;
+      if (i < 96 && c < 3 * op.nP) Zc[offP + c] = x[offP + c];
+    } else {
+      const int c = 64 * (b - op.gU - op.gP) + (i & 63);
+      const size_t o = (i < 64 ? offX : offL) + c;
+      if (c < 2 * op.nS) Zc[o] = x[o];
+    }
+  }
   if (b < op.gU) {
     const int r = b * 32 + wrow;
     const bool live = r < op.nU;
@@ -699,14 +716,14 @@ __device__ __forceinline__ double block_sum(double v, double* sm) {
 // returns true in the last block to finish (after its partial is visible)
 __device__ __forceinline__ bool last_block(unsigned int* counter) {
   __shared__ bool is_last;
-  __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
+    __threadfence();   // cumulative: covers the CTA's writes ordered before the barrier
     const unsigned int t = atomicAdd(counter, 1u);
     is_last = (t == gridDim.x - 1);
+    __threadfence();
   }
   __syncthreads();
-  if (is_last) __threadfence();
   return is_last;
 }
 

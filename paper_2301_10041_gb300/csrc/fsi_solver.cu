@@ -1147,70 +1147,155 @@ static void precond_launch(Problem& P, Prec<T>& pr, cudaStream_t s) {
 }
 
 // --------------------------------------------------------- Krylov kernels
-// Reductions over the n unknowns use a fixed grid of nb CTAs of 256 threads,
-// CTA b owning rows [512 b, 512 b + 512); per-CTA partials are summed in a
-// fixed order, so every result is deterministic.  On GB300 these kernels are
-// bound by the FP64 pipe (2 DFMA per clock per SM), so the multi-dot gives
-// each warp whole vectors and each lane 16 rows of a vector: 16 DFMA against
-// the 8 DADD of its partial sums and warp shuffle.
-constexpr int kChunk = 512;
+// Reductions over the n unknowns use a fixed grid of nb CTAs of 256 threads;
+// CTA b owns the sub-chunks b, b + nb, ... of CH rows, and the per-CTA partials
+// are summed in a fixed order, so every result is deterministic.  n is even
+// (three of the four segments are pairs and N is even), so every column of V
+// starts on a 16-byte boundary and rows are taken in pairs.
+//
+// On GB300 these kernels are bound by the FP64 pipe (2 DFMA per clock per SM)
+// when n is large, and by their chain of dependent round trips when it is
+// small.  The multi-dot gives each warp whole vectors (eight 16-byte loads in
+// flight per lane, one shuffle reduction per four vectors and CH rows).  At
+// most kRedMaxBlocks CTAs write partials, so the last CTA sums at most 32
+// values per lane and vector; with one partial per 512 rows that sum alone
+// took 40 of the 186 us of pass 1 at N = 512.
+constexpr int kRedMaxBlocks = 1024;
+constexpr int kChunkSmall = 512;     // rows per sub-chunk up to 2^19 unknowns
+constexpr int kChunkLarge = 1024;    // beyond: half as many shuffle reductions
+static inline int red_chunk(size_t n) { return n <= ((size_t)1 << 19) ? kChunkSmall : kChunkLarge; }
+static inline int red_grid(size_t n) {
+  const size_t nsub = (n + red_chunk(n) - 1) / red_chunk(n);
+  const size_t rounds = (nsub + kRedMaxBlocks - 1) / kRedMaxBlocks;
+  return (int)((nsub + rounds - 1) / rounds);
+}
 
-__device__ void mdot_warps(const double* __restrict__ V, size_t ld, int cnt, const double* __restrict__ ws, int r0,
-                           int nrow, double* __restrict__ part, int nb) {
-  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int i = wp; i < cnt; i += nw) {
-    const double* __restrict__ v = V + (size_t)i * ld + r0;
-    double a0 = 0, a1 = 0, a2 = 0, a3 = 0;
-    if (nrow == kChunk) {
+// Sums of a, b, c, d over the warp, in lanes 0, 8, 16, 24: the four share the
+// steps of one butterfly (6 additions, where four separate sums take 20; an
+// FP64 instruction holds its pipe for 64 cycles on this part).
+__device__ __forceinline__ double warp_sum4(double a, double b, double c, double d) {
+  const int lane = threadIdx.x & 31;
+  const bool hi = lane & 16, h8 = lane & 8;
+  const double s0 = (hi ? c : a) + __shfl_xor_sync(0xffffffffu, hi ? a : c, 16);
+  const double s1 = (hi ? d : b) + __shfl_xor_sync(0xffffffffu, hi ? b : d, 16);
+  double s = (h8 ? s1 : s0) + __shfl_xor_sync(0xffffffffu, h8 ? s0 : s1, 8);
 #pragma unroll
-      for (int q = 0; q < kChunk / 128; ++q) {
-        const int r = lane + 128 * q;
-        a0 += v[r] * ws[r];
-        a1 += v[r + 32] * ws[r + 32];
-        a2 += v[r + 64] * ws[r + 64];
-        a3 += v[r + 96] * ws[r + 96];
+  for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
+// this lane's part of V[i] . ws over CH rows (nrow of them in the last chunk)
+template <int CH>
+__device__ __forceinline__ double dot_part(const double* __restrict__ v, const double* __restrict__ ws, int nrow) {
+  const int lane = threadIdx.x & 31;
+  const double2* __restrict__ v2 = reinterpret_cast<const double2*>(v);
+  const double2* __restrict__ w2 = reinterpret_cast<const double2*>(ws);
+  double a0 = 0, a1 = 0;
+  if (nrow == CH) {
+#pragma unroll
+    for (int h = 0; h < CH / 512; ++h) {
+      double2 x[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) x[q] = v2[lane + 32 * (8 * h + q)];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const double2 w = w2[lane + 32 * (8 * h + q)];
+        a0 += x[q].x * w.x;
+        a1 += x[q].y * w.y;
       }
-    } else {
-      for (int r = lane; r < nrow; r += 32) a0 += v[r] * ws[r];
     }
-    const double sa = warp_sum((a0 + a1) + (a2 + a3));
-    if (lane == 0) part[(size_t)i * nb + blockIdx.x] = sa;
+  } else {
+    for (int r = lane; 2 * r < nrow; r += 32) {
+      const double2 x = v2[r], w = w2[r];
+      a0 += x.x * w.x;
+      a1 += x.y * w.y;
+    }
+  }
+  return a0 + a1;
+}
+
+// acc[i] += V[i] . ws over the nrow rows from r0 (ws: nrow values in shared
+// memory); warp w of the eight takes the vectors w, w + 8, ..., and only it
+// touches their acc[i]
+template <int CH>
+__device__ __forceinline__ void mdot_warps(const double* __restrict__ V, size_t ld, int cnt,
+                                           const double* __restrict__ ws, size_t r0, int nrow,
+                                           double* __restrict__ acc) {
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  for (int i = wp; i < cnt; i += 32) {
+    double a[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (i + 8 * q < cnt) a[q] = dot_part<CH>(V + (size_t)(i + 8 * q) * ld + r0, ws, nrow);
+    const double s = warp_sum4(a[0], a[1], a[2], a[3]);
+    const int mine = i + (lane & 24);
+    if ((lane & 7) == 0 && mine < cnt) acc[mine] += s;
   }
 }
 
-__device__ void finalize_warps(const double* __restrict__ part, int nb, int cnt, double* __restrict__ out) {
-  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int i = wp; i < cnt; i += nw) {
-    double acc = 0;
-    for (int b = lane; b < nb; b += 32) acc += part[(size_t)i * nb + b];
-    acc = warp_sum(acc);
-    if (lane == 0) out[i] = acc;
+// out[i] = sum over the nb CTAs of part[i nb + b]
+__device__ __forceinline__ void finalize_warps(const double* __restrict__ part, int nb, int cnt,
+                                               double* __restrict__ out) {
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  for (int i = wp; i < cnt; i += 32) {
+    const double* __restrict__ p = part + (size_t)i * nb;
+    double a[4] = {0, 0, 0, 0};
+#pragma unroll 4
+    for (int b = lane; b < nb; b += 32) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (i + 8 * q < cnt) a[q] += p[(size_t)(8 * q) * nb + b];
+    }
+    const double s = warp_sum4(a[0], a[1], a[2], a[3]);
+    const int mine = i + (lane & 24);
+    if ((lane & 7) == 0 && mine < cnt) out[mine] = s;
   }
 }
 
-// w[r] - sum_i V[i][r] h[i] with four independent partial sums
-__device__ __forceinline__ double gs_update(const double* __restrict__ V, size_t ld, int cnt, const double* hs,
-                                            double w, int r) {
-  double s0 = 0, s1 = 0, s2 = 0, s3 = 0;
+// w - sum_i V[i] h[i] at the row pair r2 (rows 2 r2, 2 r2 + 1), eight columns
+// in flight
+__device__ __forceinline__ double2 gs_update(const double* __restrict__ V, size_t ld, int cnt, const double* hs,
+                                             double2 w, size_t r2) {
+  const double2* __restrict__ v = reinterpret_cast<const double2*>(V) + r2;
+  const size_t l2 = ld >> 1;
+  double s0 = 0, s1 = 0, t0 = 0, t1 = 0;
   int i = 0;
-  for (; i + 3 < cnt; i += 4) {
-    s0 += V[(size_t)i * ld + r] * hs[i];
-    s1 += V[(size_t)(i + 1) * ld + r] * hs[i + 1];
-    s2 += V[(size_t)(i + 2) * ld + r] * hs[i + 2];
-    s3 += V[(size_t)(i + 3) * ld + r] * hs[i + 3];
+  for (; i + 7 < cnt; i += 8) {
+    double2 x[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) x[q] = v[(size_t)(i + q) * l2];
+#pragma unroll
+    for (int q = 0; q < 8; q += 2) {
+      s0 += x[q].x * hs[i + q];
+      s1 += x[q].y * hs[i + q];
+      t0 += x[q + 1].x * hs[i + q + 1];
+      t1 += x[q + 1].y * hs[i + q + 1];
+    }
   }
-  for (; i < cnt; ++i) s0 += V[(size_t)i * ld + r] * hs[i];
-  return w - ((s0 + s1) + (s2 + s3));
+  if (i < cnt) {   // up to seven more, still all in flight at once
+    double2 x[8];
+#pragma unroll
+    for (int q = 0; q < 7; ++q)
+      if (i + q < cnt) x[q] = v[(size_t)(i + q) * l2];
+#pragma unroll
+    for (int q = 0; q < 7; ++q)
+      if (i + q < cnt) {
+        s0 += x[q].x * hs[i + q];
+        s1 += x[q].y * hs[i + q];
+      }
+  }
+  w.x -= s0 + t0;
+  w.y -= s1 + t1;
+  return w;
 }
 
 struct KrylovArgs {
   int n;
-  int chunk;
+  int chunk;     // rows per sub-chunk of the reductions (red_chunk)
   size_t ld;
   const double* V;
   double* w;
-  double* part;
-  int pstride;   // unused by the partial layout part[i * nb + block]
+  double* part;  // part[i * nb + block]
   double* h1;
   double* h2;
   double* H;
@@ -1224,164 +1309,239 @@ struct KrylovArgs {
 
 // Classical Gram-Schmidt with one refinement pass when needed (Daniel,
 // Gragg, Kaufman and Stewart 1976; the "refine if needed" rule of PETSc's
-// GMRES): pass 1 forms h1 = V^T w and ||w||; pass 2 updates w -= V h1 and
-// forms ||w||; if the norm fell below ||w|| / sqrt(2), passes 3-4 repeat the
-// projection (h2 = V^T w, w -= V h2).  Passes 3-4 return at once otherwise.
+// GMRES): pass 1 forms h1 = V^T w and ||w||; pass 2 updates w -= V h1, forms
+// ||w|| and already the second projection h2 = V^T w, while the CTA's part
+// of V is still in its L1; if the norm fell below ||w|| / sqrt(2), pass 3
+// subtracts w -= V h2 (it returns at once otherwise).  Forming h2 in pass 2
+// replaces a pass of its own (launch, reduction and a third read of V) in
+// the refined steps, which a preconditioner that works makes the common ones:
+// A z_j is then close to v_j and most of w cancels.
 
 // Hessenberg column j, Givens rotation, residual estimate and the stop
-// decision of the Arnoldi loop (one thread)
-__device__ void arnoldi_finish(const KrylovArgs& k, double s2) {
-  Ctl* c = k.ctl;
-  const int j = c->j, m1 = c->m + 1;
-  double* Hc = k.H + (size_t)j * m1;
-  for (int i = 0; i <= j; ++i) Hc[i] = k.h1[i] + (c->refine ? k.h2[i] : 0.0);
-  const double nrm = sqrt(s2);
-  Hc[j + 1] = nrm;
-  for (int i = 0; i < j; ++i) {
-    const double a = Hc[i], b = Hc[i + 1];
-    Hc[i] = k.cs[i] * a + k.sn[i] * b;
-    Hc[i + 1] = -k.sn[i] * a + k.cs[i] * b;
-  }
-  const double a = Hc[j], b = Hc[j + 1];
-  const double r = hypot(a, b);
-  const double cc = (r > 0) ? a / r : 1.0, ss = (r > 0) ? b / r : 0.0;
-  k.cs[j] = cc; k.sn[j] = ss;
-  Hc[j] = r; Hc[j + 1] = 0.0;
-  k.g[j + 1] = -ss * k.g[j];
-  k.g[j] = cc * k.g[j];
-  const double res = fabs(k.g[j + 1]);
-  c->its += 1;
-  c->res = res;
-  bool stop = false;
-  if (!(res == res) || !(nrm == nrm)) { c->flags |= FLAG_NAN; stop = true; c->j = j; }
-  else if (r == 0.0) { c->flags |= FLAG_BREAKDOWN; stop = true; c->j = j; }
-  else {
-    c->j = j + 1;
-    if (res <= c->cycle_tol || j + 1 >= c->m || c->its >= c->max_it || nrm == 0.0) stop = true;
-  }
-  c->scale = (nrm > 0.0) ? 1.0 / nrm : 0.0;
-  c->cyc_active = stop ? 0 : 1;
-  if (k.cond) cudaGraphSetConditional(k.cond, stop ? 0u : 1u);
-}
+// decision of the Arnoldi loop, by one whole CTA.  An FP64 instruction of a
+// warp holds its pipe for 64 cycles here whatever its active lanes, so what
+// does not depend on the recurrence runs on all lanes at once: of the earlier
+// rotations only a' = c b - s a is a chain (one multiply-add per rotation, the
+// products c b formed before, the rotated entries after), the two square roots
+// share one instruction sequence and so do the three quotients.  Written for
+// one thread with every step a global read, a hypot and three divisions, this
+// made pass 2 15 us at N = 16, where its data is nothing.  Pass 1 / pass 2 or 4
+// / the least squares at j = 10 went from 10.7 / 15.3 / 10 to 7.2 / 13 / 2.7 us
+// at N = 24 (pass 2 now with the second projection), from 186 / 138 / - to 119 /
+// 228 us at N = 512, where the former pass 3 took 159.
+struct ArnoldiShared {
+  double h[256], cb[256], ns[256], a[256];   // column, c b, -s, partly rotated a
+};
 
-// pass 1: h1 = V[0..j]^T w and ||w||^2 (w is stored as vector j+1 of the dots)
-__global__ void __launch_bounds__(kRedThreads) k_gs1(KrylovArgs k) {
-  pdl_begin();
-  __shared__ double ws[kChunk];
-  __shared__ double sm[32];
-  const int cnt = k.ctl->j + 1;
-  const int r0 = blockIdx.x * kChunk, r1 = min(k.n, r0 + kChunk);
-  double acc = 0;
-  for (int r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
-    const double v = k.w[r];
-    ws[r - r0] = v;
-    acc += v * v;
+__device__ __forceinline__ void arnoldi_finish(const KrylovArgs& k, ArnoldiShared& sh, const double* h2s, double s2) {
+  Ctl* c = k.ctl;
+  const int j = c->j, m1 = c->m + 1, t = threadIdx.x;   // j < 250 <= the CTA's threads
+  double cst = 0, snt = 0;
+  if (t <= j) sh.h[t] = k.h1[t] + (h2s ? h2s[t] : 0.0);
+  if (t < j) {
+    cst = k.cs[t];
+    snt = k.sn[t];
+    sh.ns[t] = -snt;
   }
-  acc = block_sum(acc, sm);
-  if (threadIdx.x == 0) k.part[(size_t)cnt * gridDim.x + blockIdx.x] = acc;
   __syncthreads();
-  mdot_warps(k.V, k.ld, cnt, ws, r0, r1 - r0, k.part, gridDim.x);
-  if (last_block(&k.ctl->counter[0])) {
-    finalize_warps(k.part, gridDim.x, cnt + 1, k.h1);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      k.ctl->wnorm2 = k.h1[cnt];
-      k.ctl->counter[0] = 0;
+  if (t < j) sh.cb[t] = cst * sh.h[t + 1];
+  __syncthreads();
+  if (t < 32) {
+    double a = sh.h[0];
+    for (int i = 0; i < j; ++i) {
+      if (t == 0) sh.a[i] = a;
+      a = fma(sh.ns[i], a, sh.cb[i]);
+    }
+    // r = sqrt(a^2 + ||w||^2) in lane 0, ||w|| in lane 1
+    const double root = sqrt(t == 0 ? fma(a, a, s2) : s2);
+    const double r = __shfl_sync(0xffffffffu, root, 0), nrm = __shfl_sync(0xffffffffu, root, 1);
+    // a / r, ||w|| / r, 1 / ||w||
+    const double quo = (t == 0 ? a : (t == 1 ? nrm : 1.0)) / (t <= 1 ? r : nrm);
+    const double q0 = __shfl_sync(0xffffffffu, quo, 0), q1 = __shfl_sync(0xffffffffu, quo, 1);
+    const double q2 = __shfl_sync(0xffffffffu, quo, 2);
+    if (t == 0) {
+      const double gj = k.g[j];
+      const double cc = (r > 0) ? q0 : 1.0, ss = (r > 0) ? q1 : 0.0;
+      k.cs[j] = cc;
+      k.sn[j] = ss;
+      const double gn = -ss * gj;
+      k.g[j + 1] = gn;
+      k.g[j] = cc * gj;
+      k.H[(size_t)j * m1 + j] = r;
+      k.H[(size_t)j * m1 + j + 1] = 0.0;
+      const double res = fabs(gn);
+      const int its = c->its + 1;
+      c->its = its;
+      c->res = res;
+      bool stop = false;
+      if (!(res == res) || !(nrm == nrm)) { c->flags |= FLAG_NAN; stop = true; c->j = j; }
+      else if (r == 0.0) { c->flags |= FLAG_BREAKDOWN; stop = true; c->j = j; }
+      else {
+        c->j = j + 1;
+        if (res <= c->cycle_tol || j + 1 >= c->m || its >= c->max_it || nrm == 0.0) stop = true;
+      }
+      c->scale = (nrm > 0.0) ? q2 : 0.0;
+      c->cyc_active = stop ? 0 : 1;
+      if (k.cond) cudaGraphSetConditional(k.cond, stop ? 0u : 1u);
     }
   }
+  __syncthreads();
+  if (t < j) k.H[(size_t)j * m1 + t] = cst * sh.a[t] + snt * sh.h[t + 1];
 }
 
-// pass 2: w -= V h1 and ||w||^2; finish the step or ask for refinement
-__global__ void __launch_bounds__(kRedThreads) k_gs2(KrylovArgs k) {
+// rows of sub-chunk `sub` into ws (shared); the number of rows
+template <int CH>
+__device__ __forceinline__ int load_chunk(const KrylovArgs& k, int sub, double* ws) {
+  const size_t r0 = (size_t)sub * CH;
+  const int nrow = (int)min((size_t)CH, (size_t)k.n - r0);
+  const double2* __restrict__ w = reinterpret_cast<const double2*>(k.w + r0);
+  for (int r = threadIdx.x; 2 * r < nrow; r += blockDim.x) reinterpret_cast<double2*>(ws)[r] = w[r];
+  return nrow;
+}
+
+// pass 1: h1 = V[0..j]^T w and ||w||^2
+template <int CH>
+__global__ void __launch_bounds__(kRedThreads, 3) k_gs1(KrylovArgs k) {
   pdl_begin();
-  __shared__ double hs[256];
-  __shared__ double sm[32];
-  const int cnt = k.ctl->j + 1;
-  for (int i = threadIdx.x; i < cnt; i += blockDim.x) hs[i] = k.h1[i];
-  __syncthreads();
-  const int r0 = blockIdx.x * kChunk, r1 = min(k.n, r0 + kChunk);
-  double acc = 0;
-  for (int r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
-    const double v = gs_update(k.V, k.ld, cnt, hs, k.w[r], r);
-    k.w[r] = v;
-    acc += v * v;
+  __shared__ __align__(16) double ws[CH];
+  __shared__ double acc[256 + 1];
+  const int cnt = k.ctl->j + 1, nb = gridDim.x;
+  for (int i = threadIdx.x; i <= cnt; i += blockDim.x) acc[i] = 0;
+  const int nsub = (k.n + CH - 1) / CH, lane = threadIdx.x & 31;
+  for (int sub = blockIdx.x; sub < nsub; sub += nb) {
+    __syncthreads();
+    const int nrow = load_chunk<CH>(k, sub, ws);
+    __syncthreads();
+    if (threadIdx.x >= kRedThreads - 32) {   // the last warp (fewest vectors): w . w
+      double a = 0;
+      for (int r = lane; r < nrow; r += 32) a += ws[r] * ws[r];
+      a = warp_sum(a);
+      if (lane == 0) acc[cnt] += a;
+    }
+    mdot_warps<CH>(k.V, k.ld, cnt, ws, (size_t)sub * CH, nrow, acc);
   }
-  acc = block_sum(acc, sm);
-  if (threadIdx.x == 0) k.part[blockIdx.x] = acc;
+  __syncthreads();
+  for (int i = threadIdx.x; i <= cnt; i += blockDim.x) k.part[(size_t)i * nb + blockIdx.x] = acc[i];
+  if (last_block(&k.ctl->counter[0])) {
+    finalize_warps(k.part, nb, cnt + 1, k.h1);
+    if (threadIdx.x == 0) k.ctl->counter[0] = 0;
+  }
+}
+
+// pass 2: w -= V h1, ||w||^2 and h2 = V^T w; finish the step or ask for the
+// refinement (h1[cnt] is ||w||^2 of pass 1)
+template <int CH>
+__global__ void __launch_bounds__(kRedThreads, 3) k_gs2(KrylovArgs k) {
+  pdl_begin();
+  __shared__ __align__(16) double ws[CH];
+  __shared__ double hs[256], acc[256], sm[32];
+  __shared__ ArnoldiShared ash;
+  __shared__ double s2s;
+  const int cnt = k.ctl->j + 1, nb = gridDim.x;
+  for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
+    hs[i] = k.h1[i];
+    acc[i] = 0;
+  }
+  const int nsub = (k.n + CH - 1) / CH;
+  double nacc = 0;
+  for (int sub = blockIdx.x; sub < nsub; sub += nb) {
+    __syncthreads();
+    const size_t r0 = (size_t)sub * CH;
+    const int nrow = (int)min((size_t)CH, (size_t)k.n - r0);
+    double2* w2 = reinterpret_cast<double2*>(k.w + r0);
+    for (int r = threadIdx.x; 2 * r < nrow; r += blockDim.x) {
+      const double2 v = gs_update(k.V, k.ld, cnt, hs, w2[r], (r0 >> 1) + r);
+      w2[r] = v;
+      reinterpret_cast<double2*>(ws)[r] = v;
+      nacc += v.x * v.x + v.y * v.y;
+    }
+    __syncthreads();
+    mdot_warps<CH>(k.V, k.ld, cnt, ws, r0, nrow, acc);
+  }
+  const double bs = block_sum(nacc, sm);
+  if (threadIdx.x == 0) k.part[(size_t)cnt * nb + blockIdx.x] = bs;
+  for (int i = threadIdx.x; i < cnt; i += blockDim.x) k.part[(size_t)i * nb + blockIdx.x] = acc[i];
   if (last_block(&k.ctl->counter[1])) {
-    double a = 0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) a += k.part[b];
-    const double s2 = block_sum(a, sm);
+    finalize_warps(k.part, nb, cnt + 1, k.h2);
+    __syncthreads();
     if (threadIdx.x == 0) {
       Ctl* c = k.ctl;
       c->counter[1] = 0;
-      c->refine = (s2 < 0.5 * c->wnorm2) ? 1 : 0;
+      const double s2 = k.h2[cnt];
+      c->refine = (s2 < 0.5 * k.h1[cnt]) ? 1 : 0;
       if (c->refine) c->refines += 1;
-      else arnoldi_finish(k, s2);
+      s2s = c->refine ? -1.0 : s2;
     }
+    __syncthreads();
+    // -1 marks the refinement; a NaN norm is not below any bound and finishes here
+    if (s2s != -1.0) arnoldi_finish(k, ash, nullptr, s2s);
   }
 }
 
-// pass 3 (refinement only): h2 = V^T w
-__global__ void __launch_bounds__(kRedThreads) k_gs3(KrylovArgs k) {
+// pass 3 (refinement only): w -= V h2, ||w||^2, finish the step
+template <int CH>
+__global__ void __launch_bounds__(kRedThreads, 3) k_gs3(KrylovArgs k) {
   pdl_begin();
-  __shared__ double ws[kChunk];
+  __shared__ double hs[256], sm[32];
+  __shared__ ArnoldiShared ash;
+  __shared__ double s2s;
   if (!k.ctl->refine) return;
-  const int cnt = k.ctl->j + 1;
-  const int r0 = blockIdx.x * kChunk, r1 = min(k.n, r0 + kChunk);
-  for (int r = r0 + threadIdx.x; r < r1; r += blockDim.x) ws[r - r0] = k.w[r];
-  __syncthreads();
-  mdot_warps(k.V, k.ld, cnt, ws, r0, r1 - r0, k.part, gridDim.x);
-  if (last_block(&k.ctl->counter[2])) {
-    finalize_warps(k.part, gridDim.x, cnt, k.h2);
-    if (threadIdx.x == 0) k.ctl->counter[2] = 0;
-  }
-}
-
-// pass 4 (refinement only): w -= V h2, ||w||^2, finish the step
-__global__ void __launch_bounds__(kRedThreads) k_gs4(KrylovArgs k) {
-  pdl_begin();
-  __shared__ double hs[256];
-  __shared__ double sm[32];
-  if (!k.ctl->refine) return;
-  const int cnt = k.ctl->j + 1;
+  const int cnt = k.ctl->j + 1, nb = gridDim.x;
   for (int i = threadIdx.x; i < cnt; i += blockDim.x) hs[i] = k.h2[i];
   __syncthreads();
-  const int r0 = blockIdx.x * kChunk, r1 = min(k.n, r0 + kChunk);
-  double acc = 0;
-  for (int r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
-    const double v = gs_update(k.V, k.ld, cnt, hs, k.w[r], r);
-    k.w[r] = v;
-    acc += v * v;
+  const int nsub = (k.n + CH - 1) / CH;
+  double nacc = 0;
+  for (int sub = blockIdx.x; sub < nsub; sub += nb) {
+    const size_t r0 = (size_t)sub * CH;
+    const int nrow = (int)min((size_t)CH, (size_t)k.n - r0);
+    double2* w2 = reinterpret_cast<double2*>(k.w + r0);
+    for (int r = threadIdx.x; 2 * r < nrow; r += blockDim.x) {
+      const double2 v = gs_update(k.V, k.ld, cnt, hs, w2[r], (r0 >> 1) + r);
+      w2[r] = v;
+      nacc += v.x * v.x + v.y * v.y;
+    }
   }
-  acc = block_sum(acc, sm);
-  if (threadIdx.x == 0) k.part[blockIdx.x] = acc;
-  if (last_block(&k.ctl->counter[6])) {
+  const double bs = block_sum(nacc, sm);
+  if (threadIdx.x == 0) k.part[blockIdx.x] = bs;
+  if (last_block(&k.ctl->counter[2])) {
     double a = 0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) a += k.part[b];
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) a += k.part[b];
     const double s2 = block_sum(a, sm);
     if (threadIdx.x == 0) {
-      k.ctl->counter[6] = 0;
-      arnoldi_finish(k, s2);
+      k.ctl->counter[2] = 0;
+      s2s = s2;
     }
+    __syncthreads();
+    arnoldi_finish(k, ash, hs, s2s);
   }
 }
 
-// V[j] = w * scale (j already advanced)
-__global__ void k_gs_scale(int n, double* __restrict__ V, size_t ld, const double* __restrict__ w, const Ctl* ctl) {
+// The next basis vector V[j] = w * scale (j already advanced, or 0 at the
+// start of a cycle), and with it the preconditioner's input in its precision.
+template <class T>
+__global__ void k_basis(int n2, double* __restrict__ V, size_t ld, const double* __restrict__ w, T* __restrict__ vin,
+                        const Ctl* ctl) {
   pdl_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  V[(size_t)ctl->j * ld + i] = w[i] * ctl->scale;
+  if (i >= n2) return;
+  const double sc = ctl->scale;
+  double2 v = reinterpret_cast<const double2*>(w)[i];
+  v.x *= sc;
+  v.y *= sc;
+  reinterpret_cast<double2*>(V + (size_t)ctl->j * ld)[i] = v;
+  typename Vec2<T>::type o;
+  o.x = (T)v.x;
+  o.y = (T)v.y;
+  reinterpret_cast<typename Vec2<T>::type*>(vin)[i] = o;
 }
 
 // start of a cycle: beta = ||w|| with w = b - A x already formed
 __global__ void __launch_bounds__(kRedThreads) k_cycle_start(KrylovArgs k) {
   pdl_begin();
   __shared__ double sm[32];
-  const int r0 = blockIdx.x * k.chunk, r1 = min(k.n, r0 + k.chunk);
   double acc = 0;
-  for (int r = r0 + threadIdx.x; r < r1; r += blockDim.x) acc += k.w[r] * k.w[r];
+  for (size_t r0 = (size_t)blockIdx.x * k.chunk; r0 < (size_t)k.n; r0 += (size_t)gridDim.x * k.chunk)
+    for (size_t r = r0 + threadIdx.x; r < min((size_t)k.n, r0 + k.chunk); r += blockDim.x) acc += k.w[r] * k.w[r];
   acc = block_sum(acc, sm);
   if (threadIdx.x == 0) k.part[blockIdx.x] = acc;
   if (last_block(&k.ctl->counter[3])) {
@@ -1414,21 +1574,14 @@ __global__ void __launch_bounds__(kRedThreads) k_cycle_start(KrylovArgs k) {
   }
 }
 
-__global__ void k_scale0(int n, double* __restrict__ V, const double* __restrict__ w, const Ctl* ctl) {
-  pdl_begin();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  V[i] = w[i] * ctl->scale;
-}
-
 // ||b||, the target, and reset of the per-solve counters
 __global__ void __launch_bounds__(kRedThreads) k_solve_begin(KrylovArgs k, const double* __restrict__ b, double rtol,
                                                              double inner_rtol, int max_it, int m, int max_cycles) {
   pdl_begin();
   __shared__ double sm[32];
-  const int r0 = blockIdx.x * k.chunk, r1 = min(k.n, r0 + k.chunk);
   double acc = 0;
-  for (int r = r0 + threadIdx.x; r < r1; r += blockDim.x) acc += b[r] * b[r];
+  for (size_t r0 = (size_t)blockIdx.x * k.chunk; r0 < (size_t)k.n; r0 += (size_t)gridDim.x * k.chunk)
+    for (size_t r = r0 + threadIdx.x; r < min((size_t)k.n, r0 + k.chunk); r += blockDim.x) acc += b[r] * b[r];
   acc = block_sum(acc, sm);
   if (threadIdx.x == 0) k.part[blockIdx.x] = acc;
   if (last_block(&k.ctl->counter[4])) {
@@ -1448,44 +1601,85 @@ __global__ void __launch_bounds__(kRedThreads) k_solve_begin(KrylovArgs k, const
   }
 }
 
-// least squares on the rotated Hessenberg matrix: y = R^-1 g (one thread)
-__global__ void k_lsq(const double* __restrict__ H, const double* __restrict__ g, double* __restrict__ y,
-                      const Ctl* ctl) {
+// least squares on the rotated Hessenberg matrix: y = R^-1 g by one warp.
+// Column-oriented back substitution: lane l holds the right-hand sides l,
+// l + 32, ... and the reciprocals of their diagonals (all taken at once); each
+// solved entry is broadcast and its column, the next one already loading,
+// subtracted from the entries above.  So a step is one multiplication and one
+// multiply-add deep.  (One thread walking the rows, with a dependent global
+// read per entry and a division per row, took 10 us at 10 entries.)
+constexpr int kLsqRows = 8;   // 32 * 8 >= the largest restart
+__global__ void __launch_bounds__(32) k_lsq(const double* __restrict__ H, const double* __restrict__ g,
+                                            double* __restrict__ y, const Ctl* ctl) {
   pdl_begin();
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+  const int lane = threadIdx.x;
   const int kk = ctl->j, m1 = ctl->m + 1;
-  for (int i = kk - 1; i >= 0; --i) {
-    double v = g[i];
-    for (int l = i + 1; l < kk; ++l) v -= H[(size_t)l * m1 + i] * y[l];
-    y[i] = v / H[(size_t)i * m1 + i];
+  double v[kLsqRows], inv[kLsqRows], c[kLsqRows];
+#pragma unroll
+  for (int q = 0; q < kLsqRows; ++q) {
+    const int r = lane + 32 * q;
+    v[q] = inv[q] = c[q] = 0.0;
+    if (32 * q < kk) {
+      if (r < kk) {
+        v[q] = g[r];
+        inv[q] = 1.0 / H[(size_t)r * m1 + r];
+        if (r < kk - 1) c[q] = H[(size_t)(kk - 1) * m1 + r];
+      }
+    }
+  }
+#pragma unroll
+  for (int b = kLsqRows - 1; b >= 0; --b) {
+    for (int i = min(kk, 32 * b + 32) - 1; i >= 32 * b; --i) {
+      double d[kLsqRows];   // the next column, above its diagonal
+#pragma unroll
+      for (int q = 0; q <= b; ++q) {
+        const int r = lane + 32 * q;
+        d[q] = r < i - 1 ? H[(size_t)(i - 1) * m1 + r] : 0.0;
+      }
+      const double yi = __shfl_sync(0xffffffffu, v[b] * inv[b], i & 31);
+#pragma unroll
+      for (int q = 0; q <= b; ++q) {
+        v[q] -= c[q] * yi;   // zero at and below the diagonal
+        c[q] = d[q];
+      }
+      if (lane == (i & 31)) y[i] = yi;
+    }
   }
 }
 
-// x += Z y (right preconditioning: the update lives in span{Z})
+// x += Z y (right preconditioning: the update lives in span{Z}), two rows per
+// thread, eight columns in flight
 template <class T>
-__global__ void k_xupdate(int n, double* __restrict__ x, const T* __restrict__ Z, size_t ld,
-                          const double* __restrict__ y, const Ctl* ctl) {
+__global__ void __launch_bounds__(256) k_xupdate(int n2, double* __restrict__ x, const T* __restrict__ Z, size_t ld,
+                                                 const double* __restrict__ y, const Ctl* ctl) {
   pdl_begin();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+  using T2 = typename Vec2<T>::type;
+  __shared__ double ys[256];
   const int kk = ctl->j;
-  double v = x[i];
-  for (int l = 0; l < kk; ++l) v += (double)Z[(size_t)l * ld + i] * y[l];
-  x[i] = v;
-}
-
-template <class T>
-__global__ void k_prec_in(int n, const double* __restrict__ V, size_t ld, const Ctl* ctl, T* __restrict__ vin) {
-  pdl_begin();
+  for (int l = threadIdx.x; l < kk; l += blockDim.x) ys[l] = y[l];
+  __syncthreads();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) vin[i] = (T)V[(size_t)ctl->j * ld + i];
-}
-
-template <class T>
-__global__ void k_prec_out(int n, const T* __restrict__ zw, T* __restrict__ Z, size_t ld, const Ctl* ctl) {
-  pdl_begin();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) Z[(size_t)ctl->j * ld + i] = zw[i];
+  if (i >= n2) return;
+  const T2* __restrict__ z = reinterpret_cast<const T2*>(Z) + i;
+  const size_t l2 = ld >> 1;
+  double2 v = reinterpret_cast<double2*>(x)[i];
+  int l = 0;
+  for (; l + 7 < kk; l += 8) {
+    T2 q[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) q[u] = z[(size_t)(l + u) * l2];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      v.x += (double)q[u].x * ys[l + u];
+      v.y += (double)q[u].y * ys[l + u];
+    }
+  }
+  for (; l < kk; ++l) {
+    const T2 q = z[(size_t)l * l2];
+    v.x += (double)q.x * ys[l];
+    v.y += (double)q.y * ys[l];
+  }
+  reinterpret_cast<double2*>(x)[i] = v;
 }
 
 // zero mean of the constant pressure coefficients (p in L^2_0)
@@ -1634,12 +1828,11 @@ static FullOp<T> make_op(Problem& P, const T* cfv, const T* cftv) {
 static KrylovArgs krylov_args(Problem& P, cudaGraphConditionalHandle h) {
   KrylovArgs k{};
   k.n = (int)P.n;
-  k.chunk = kChunk;
+  k.chunk = red_chunk(P.n);
   k.ld = P.n;
   k.V = P.V;
   k.w = P.w;
   k.part = P.part;
-  k.pstride = P.m + 1;
   k.h1 = P.y + (P.m + 2);       // scratch after y (m+2 entries each)
   k.h2 = P.y + 2 * (P.m + 2);
   k.H = P.H; k.cs = P.cs; k.sn = P.sn; k.g = P.g;
@@ -1686,30 +1879,38 @@ static void assemble_launch(Problem& P, cudaStream_t s) {
   sell_launch(P.Cs64, MODE_AXPBY, axpby<double>(P.Xold, P.b + P.offL, P.cflift, -1.0 / P.prm.dt, -1.0), s);
 }
 
-template <class T>
-static void iteration_launch(Problem& P, Prec<T>& pr, const KrylovArgs& k, cudaStream_t s) {
-  const unsigned gn = nblk(P.n, 256);
-  launch(k_prec_in<T>, gn, 256, 0, s, (int)P.n, P.V, P.n, P.ctl, pr.vin);
-  precond_launch(P, pr, s);
-  launch(k_prec_out<T>, gn, 256, 0, s, (int)P.n, pr.zw, (T*)P.Z, P.n, P.ctl);
-  launch(k_fullmv<T, T, double>, pr.op.gU + pr.op.gP + pr.op.gS, 128, 0, s, pr.op, pr.zw, P.w, nullptr, 1.0, 0.0);
-  launch(k_gs1, P.red_blocks, kRedThreads, 0, s, k);
-  launch(k_gs2, P.red_blocks, kRedThreads, 0, s, k);
-  launch(k_gs3, P.red_blocks, kRedThreads, 0, s, k);
-  launch(k_gs4, P.red_blocks, kRedThreads, 0, s, k);
-  launch(k_gs_scale, gn, 256, 0, s, (int)P.n, P.V, P.n, P.w, P.ctl);
+// Gram-Schmidt of w against V[0..j], the Givens step and the next basis vector
+template <int CH, class T>
+static void orthogonalise_launch(Problem& P, Prec<T>& pr, const KrylovArgs& k, cudaStream_t s) {
+  launch(k_gs1<CH>, P.red_blocks, kRedThreads, 0, s, k);
+  launch(k_gs2<CH>, P.red_blocks, kRedThreads, 0, s, k);
+  launch(k_gs3<CH>, P.red_blocks, kRedThreads, 0, s, k);
+  launch(k_basis<T>, nblk(P.n / 2, 256), 256, 0, s, (int)(P.n / 2), P.V, P.n, P.w, pr.vin, P.ctl);
 }
 
-static void cycle_start_launch(Problem& P, const KrylovArgs& k, cudaStream_t s) {
-  launch(k_fullmv<double, double, double>, P.op64.gU + P.op64.gP + P.op64.gS, 128, 0, s, P.op64, P.x, P.w, P.b, -1.0, 1.0);
+// One Arnoldi iteration; pr.vin holds v_j on entry (k_basis of the previous
+// iteration or of the cycle's start wrote it).
+template <class T>
+static void iteration_launch(Problem& P, Prec<T>& pr, const KrylovArgs& k, cudaStream_t s) {
+  precond_launch(P, pr, s);
+  launch(k_fullmv<T, T, double>, pr.op.gU + pr.op.gP + pr.op.gS, 128, 0, s, pr.op, pr.zw, P.w, nullptr, 1.0, 0.0,
+         (T*)P.Z, P.n, (const Ctl*)P.ctl);
+  if (k.chunk == kChunkSmall) orthogonalise_launch<kChunkSmall>(P, pr, k, s);
+  else orthogonalise_launch<kChunkLarge>(P, pr, k, s);
+}
+
+template <class T>
+static void cycle_start_launch(Problem& P, Prec<T>& pr, const KrylovArgs& k, cudaStream_t s) {
+  launch(k_fullmv<double, double, double>, P.op64.gU + P.op64.gP + P.op64.gS, 128, 0, s, P.op64, P.x, P.w, P.b, -1.0,
+         1.0, (double*)nullptr, (size_t)0, (const Ctl*)nullptr);
   launch(k_cycle_start, P.red_blocks, kRedThreads, 0, s, k);
-  launch(k_scale0, nblk(P.n, 256), 256, 0, s, (int)P.n, P.V, P.w, P.ctl);
+  launch(k_basis<T>, nblk(P.n / 2, 256), 256, 0, s, (int)(P.n / 2), P.V, P.n, P.w, pr.vin, P.ctl);
 }
 
 template <class T>
 static void cycle_end_launch(Problem& P, cudaStream_t s) {
   launch(k_lsq, 1, 32, 0, s, P.H, P.g, P.y, P.ctl);
-  launch(k_xupdate<T>, nblk(P.n, 256), 256, 0, s, (int)P.n, P.x, (const T*)P.Z, P.n, P.y, P.ctl);
+  launch(k_xupdate<T>, nblk(P.n / 2, 256), 256, 0, s, (int)(P.n / 2), P.x, (const T*)P.Z, P.n, P.y, P.ctl);
 }
 
 static int count_kernel_nodes(cudaGraph_t g) {
@@ -1728,7 +1929,7 @@ static int count_kernel_nodes(cudaGraph_t g) {
 
 // The whole solve as one graph: an outer WHILE node over restart/refinement
 // cycles whose body computes the true FP64 residual (k_cycle_start sets both
-// conditions), runs the Arnoldi loop as an inner WHILE node (k_gs2/k_gs4 set
+// conditions), runs the Arnoldi loop as an inner WHILE node (k_gs2/k_gs3 set
 // its condition) and updates x.  No host round trip inside a solve.
 template <class T>
 static void build_cycle_graph(Problem& P, Prec<T>& pr) {
@@ -1750,7 +1951,7 @@ static void build_cycle_graph(Problem& P, Prec<T>& pr) {
   CK(cudaGraphConditionalHandleCreate(&h_in, obody, 0, 0));
   KrylovArgs k = krylov_args(P, h_in);
   k.cond_outer = h_out;
-  cycle_start_launch(P, k, s);
+  cycle_start_launch(P, pr, k, s);
   cudaStreamCaptureStatus st;
   cudaGraph_t cg = nullptr;
   const cudaGraphNode_t* deps = nullptr;
@@ -1783,7 +1984,7 @@ static void build_host_loop_graphs(Problem& P, Prec<T>& pr) {
   cudaStream_t s = P.stream;
   KrylovArgs k = krylov_args(P, 0);
   CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-  cycle_start_launch(P, k, s);
+  cycle_start_launch(P, pr, k, s);
   CK(cudaStreamEndCapture(s, &P.gr_cstart));
   CK(cudaGraphInstantiate(&P.g_cstart, P.gr_cstart, 0));
   CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
@@ -1922,7 +2123,7 @@ static void allocate_problem(Problem& P, const double* ref_xy, const int* tris_h
   P.sn = ar.alloc<double>(m + 1);
   P.g = ar.alloc<double>(m + 2);
   P.y = ar.alloc<double>(3 * (size_t)(m + 2));
-  P.red_blocks = (int)((P.n + kChunk - 1) / kChunk);
+  P.red_blocks = red_grid(P.n);
   P.part = ar.alloc<double>((size_t)std::max(P.red_blocks, 64) * (m + 2));
   P.ctl = ar.alloc<Ctl>(1);
   P.op64 = make_op<double>(P, P.cf_val, P.cft_val);
@@ -2511,10 +2712,10 @@ int fsi_apply_operator(fsi_problem* h, const double* xh, double* yh, int precisi
     if (precision == 1) {
       launch(k_convert<double, float>, nblk(P.n, 256), 256, 0, P.stream, P.n, tmp, P.p32.vin);
       launch(k_fullmv<float, float, double>, P.op32.gU + P.op32.gP + P.op32.gS, 128, 0, P.stream, P.op32, P.p32.vin, P.w,
-                                                                                            nullptr, 1.0, 0.0);
+             nullptr, 1.0, 0.0, (float*)nullptr, (size_t)0, (const Ctl*)nullptr);
     } else {
       launch(k_fullmv<double, double, double>, P.op64.gU + P.op64.gP + P.op64.gS, 128, 0, P.stream, P.op64, tmp, P.w,
-                                                                                               nullptr, 1.0, 0.0);
+             nullptr, 1.0, 0.0, (double*)nullptr, (size_t)0, (const Ctl*)nullptr);
     }
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(yh, P.w, P.n * 8, cudaMemcpyDeviceToHost, P.stream));
@@ -2588,12 +2789,12 @@ int fsi_time_kernel(fsi_problem* h, int which, int reps, double* avg_ms, double*
       switch (which) {
         case 0:  // full operator, FP32 (mixed inner iteration)
           launch(k_fullmv<float, float, double>, P.op32.gU + P.op32.gP + P.op32.gS, 128, 0, s, P.op32, P.p32.zw, P.w,
-                                                                                          nullptr, 1.0, 0.0);
+                 nullptr, 1.0, 0.0, (float*)nullptr, (size_t)0, (const Ctl*)nullptr);
           *bytes = fullop_bytes<float>(P, cfnnz, sizeof(float), sizeof(double));
           break;
         case 1:  // full operator, FP64 (residual / FP64 iteration)
           launch(k_fullmv<double, double, double>, P.op64.gU + P.op64.gP + P.op64.gS, 128, 0, s, P.op64, P.x, P.w, P.b,
-                                                                                            -1.0, 1.0);
+                 -1.0, 1.0, (double*)nullptr, (size_t)0, (const Ctl*)nullptr);
           *bytes = fullop_bytes<double>(P, cfnnz, 16, 8);
           break;
         case 2: {  // finest velocity Chebyshev step, FP32
