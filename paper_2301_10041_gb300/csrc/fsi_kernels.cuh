@@ -518,22 +518,41 @@ __global__ void k_axpy(size_t n, T a, const T* __restrict__ x, T* __restrict__ y
 
 // C_f (ELL over solid nodes, kron 2) times a velocity vector:
 // y = alpha C_f u + beta z on 2 nS entries; MODE_INIT also sets d = xo = c2 dinv y.
+// Rows hold some 30 to 60 entries.  A warp takes 8 rows with 4 threads each
+// (lane = 8 t + r, so a load of one entry per row fills whole sectors), four
+// entries in flight per thread; a thread per row walked them one by one.
 template <class T>
-__global__ void k_cf_apply(int nS, int cap, const int* __restrict__ len, const int* __restrict__ col,
-                           const T* __restrict__ val, SpmvArgs<T> a, int mode) {
+__global__ void __launch_bounds__(128) k_cf_apply(int nS, int cap, const int* __restrict__ len,
+                                                  const int* __restrict__ col, const T* __restrict__ val,
+                                                  SpmvArgs<T> a, int mode) {
+  using T2 = typename Vec2<T>::type;
   pdl_begin();
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= nS) return;
+  const int lane = threadIdx.x & 31, t = lane >> 3;
+  const int r = blockIdx.x * 32 + (threadIdx.x >> 5) * 8 + (lane & 7);
+  const bool live = r < nS;
   const size_t cbase = (size_t)(r >> 5) * 32 * cap + (r & 31);
-  T a0 = 0, a1 = 0;
-  for (int k = 0; k < len[r]; ++k) {
-    const size_t slot = cbase + ((size_t)k << 5);
-    const int c = col[slot];
-    const T v = val[slot];
-    a0 += v * a.x[2 * c];
-    a1 += v * a.x[2 * c + 1];
+  T acc[2] = {0, 0};
+  const int n = live ? len[r] : 0;
+  for (int k0 = t; k0 < n; k0 += 16) {
+    int c[4];
+    T v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const size_t slot = cbase + ((size_t)(k0 + 4 * u) << 5);
+      const bool in = k0 + 4 * u < n;
+      c[u] = in ? col[slot] : 0;
+      v[u] = in ? val[slot] : (T)0;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const T2 x = reinterpret_cast<const T2*>(a.x)[c[u]];
+      acc[0] += v[u] * x.x;
+      acc[1] += v[u] * x.y;
+    }
   }
-  T t0 = a.alpha * a0, t1 = a.alpha * a1;
+  row_reduce<T, 2>(acc);
+  if (!live || t != 0) return;
+  T t0 = a.alpha * acc[0], t1 = a.alpha * acc[1];
   if (a.z) { t0 += a.beta * a.z[2 * r]; t1 += a.beta * a.z[2 * r + 1]; }
   a.y[2 * r] = t0;
   a.y[2 * r + 1] = t1;

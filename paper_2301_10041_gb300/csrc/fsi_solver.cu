@@ -33,6 +33,7 @@
 #include "fsi_kernels.cuh"
 #include "fsi_mgfused.cuh"
 #include "fsi_solid.cuh"
+#include "fsi_solid_cheb.cuh"
 
 namespace fsi {
 
@@ -834,6 +835,9 @@ struct Prec {
   T* vin = nullptr;      // preconditioner input (n)
   T* zw = nullptr;       // preconditioner output (n)
   T *sb = nullptr, *sx = nullptr, *sx2 = nullptr, *sd = nullptr;  // solid work (2 nS)
+  T* sd2 = nullptr;      // second direction buffer, when a mass solve takes several launches
+  SolidPatches<T> sc;    // patches of the mass solves (fsi_solid_cheb.cuh); np = 0: one launch per step
+  int sc_launches = 1;   // launches per mass solve
   Cheb chs;              // Chebyshev for D^-1 C_s on Wathen's interval ([1/2, 2] for P1)
   int cs_k = 16;
   // inner Richardson on the Stokes block: velocity right-hand side, residual
@@ -905,6 +909,87 @@ struct Problem {
 // bounds for the Jacobi-scaled P1 mass matrix):
 //   X = -dt C_s^-1 r_l,   lambda = C_s^-1 (A_s X - r_X),
 // with r_l = v_l - C_f z_u for the block-triangular preconditioner.
+// One mass solve C_s x = b by its patches: cs_k Chebyshev-Jacobi steps (the
+// first one the start x = d = c0 D^-1 b) over sc_launches launches.  b is
+// scale bsrc, or K kx - bsrc when kx is given.
+template <class T, int W, int RPT>
+static void solid_patch_kernel(const Prec<T>& pr, const SolidChebArgs<T>& a, cudaStream_t s) {
+  launch(k_solid_cheb<T, W, RPT, sc_threads<T>()>, pr.sc.np, sc_threads<T>(), pr.sc.smem, s, a);
+}
+
+template <class T>
+static void solid_patch_solve(Prec<T>& pr, const T* bsrc, T scale, const Sell<T>* K, const T* kx, T* out,
+                              cudaStream_t s) {
+  SolidChebArgs<T> a;
+  a.P = pr.sc;
+  a.c0 = (T)pr.chs.c0;
+  a.dinv = pr.csdinv;
+  a.bsrc = bsrc;
+  a.scale = scale;
+  if (K) a.K = *K;
+  a.kx = kx;
+  T *x[2] = {pr.sx, pr.sx2}, *d[2] = {pr.sd, pr.sd2};
+  const int m = pr.cs_k - 1;
+  int done = 0;
+  for (int l = 0; l < pr.sc_launches; ++l) {
+    a.ns = std::min(pr.sc.steps, m - done);
+    a.first = l == 0;
+    a.last = l + 1 == pr.sc_launches;
+    for (int i = 0; i < a.ns; ++i) {
+      a.c1[i] = (T)pr.chs.c1[done + i];
+      a.c2[i] = (T)pr.chs.c2[done + i];
+    }
+    done += a.ns;
+    a.xin = x[(l + 1) & 1];
+    a.din = d[(l + 1) & 1];
+    a.xout = a.last ? out : x[l & 1];
+    a.dout = d[l & 1];
+    if (pr.sc.width == 8 && pr.sc.rpt == 1) solid_patch_kernel<T, 8, 1>(pr, a, s);
+    else if (pr.sc.width == 8) solid_patch_kernel<T, 8, 2>(pr, a, s);
+    else if (pr.sc.rpt == 1) solid_patch_kernel<T, kScWide, 1>(pr, a, s);
+    else solid_patch_kernel<T, kScWide, 2>(pr, a, s);
+  }
+}
+
+// The patches of a problem's body on the device; none (np = 0) when the mesh
+// does not suit.  A footprint count without the mesh itself takes a bound.
+template <class T>
+static void setup_solid_patches(Arena& ar, const HostSetup& hs, const double* ref_xy, Prec<T>& pr) {
+  constexpr bool f64 = std::is_same<T, double>::value;
+  constexpr int NT = sc_threads<T>();
+  SolidPatchHost h;
+  if (!build_solid_patches(hs.Cs, ref_xy, pr.cs_k - 1, f64, NT, h)) {
+    if (ar.count_only) {
+      const SolidPlan pl = plan_solid_patches(hs.Cs.nrows, pr.cs_k - 1, f64, 2 * NT);
+      const double r = std::sqrt((double)hs.Cs.nrows / std::max(1, pl.np)) + 2.0 * pl.steps;
+      const double loc = pl.np * std::min((double)hs.Cs.nrows, r * r);
+      ar.bytes += (size_t)(1.3 * loc * (kScWide * (sizeof(T) + 2) + 4)) + 4096;
+    }
+    return;
+  }
+  SolidPatches<T>& d = pr.sc;
+  d.np = h.np;
+  d.steps = h.steps;
+  d.width = h.width;
+  d.rpt = h.max_rows > NT ? 2 : 1;
+  d.smem = 4 * sizeof(T) * (size_t)h.max_loc;
+  pr.sc_launches = h.launches;
+  d.poff = ar.upload(h.poff);
+  d.cnt = ar.upload(h.cnt);
+  d.gid = ar.upload(h.gid);
+  d.roff = ar.upload(h.roff);
+  d.val = upload_as<T>(ar, h.val);
+  d.col = ar.upload(h.col);
+  if (h.launches > 1) pr.sd2 = ar.alloc<T>(2 * (size_t)hs.Cs.nrows);
+  if (!ar.count_only && d.smem > 48 * 1024) {   // the limit belongs to the kernel: raise it to the cap
+    const int cap = (int)kClSmemCap;
+    CK(cudaFuncSetAttribute(k_solid_cheb<T, 8, 1, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    CK(cudaFuncSetAttribute(k_solid_cheb<T, 8, 2, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    CK(cudaFuncSetAttribute(k_solid_cheb<T, kScWide, 1, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    CK(cudaFuncSetAttribute(k_solid_cheb<T, kScWide, 2, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+  }
+}
+
 template <class T>
 static void solid_launch(Problem& P, Prec<T>& pr, cudaStream_t s) {
   const int n2 = 2 * P.nS;
@@ -914,6 +999,21 @@ static void solid_launch(Problem& P, Prec<T>& pr, cudaStream_t s) {
   T* zX = pr.zw + P.offX;
   T* zL = pr.zw + P.offL;
   const T dt = (T)P.prm.dt;
+  const unsigned gcf = nblk(P.nS, 32);
+  if (pr.sc.np > 0) {
+    const T* bsrc = vL;
+    T scale = -dt;
+    if (P.prm.precond == 1) {  // lower block-triangular: -dt (v_l - C_f z_u)
+      SpmvArgs<T> a;
+      a.x = pr.zw; a.y = pr.sb; a.z = vL; a.alpha = dt; a.beta = -dt;
+      launch(k_cf_apply<T>, gcf, 128, 0, s, P.nS, P.cf_cap, P.cf_len, P.cf_col, pr.op.cf_val, a, MODE_AXPBY);
+      bsrc = pr.sb;
+      scale = 1;
+    }
+    solid_patch_solve<T>(pr, bsrc, scale, nullptr, nullptr, zX, s);
+    solid_patch_solve<T>(pr, vX, (T)1, P.prm.solid_law == 1 ? &pr.KT : &pr.As, zX, zL, s);
+    return;
+  }
   auto cheb_rest = [&](T* out) {
     T* xc = pr.sx;
     T* xn = pr.sx2;
@@ -931,7 +1031,7 @@ static void solid_launch(Problem& P, Prec<T>& pr, cudaStream_t s) {
     SpmvArgs<T> a;
     a.x = pr.zw; a.y = pr.sb; a.z = vL; a.alpha = dt; a.beta = -dt;
     a.d = pr.sd; a.dinv = pr.csdinv; a.xo = pr.sx; a.c2 = (T)pr.chs.c0;
-    launch(k_cf_apply<T>, nblk(P.nS, 128), 128, 0, s, P.nS, P.cf_cap, P.cf_len, P.cf_col, pr.op.cf_val, a, MODE_INIT);
+    launch(k_cf_apply<T>, gcf, 128, 0, s, P.nS, P.cf_cap, P.cf_len, P.cf_col, pr.op.cf_val, a, MODE_INIT);
   } else {
     launch(k_cheb_first<T>, nblk(n2, 256), 256, 0, s, n2, vL, pr.csdinv, (T)pr.chs.c0, pr.sd, pr.sx, -dt, pr.sb);
   }
@@ -1760,8 +1860,7 @@ static fsi_params with_defaults(fsi_params p) {
 }
 
 template <class T>
-static void build_prec(Problem& P, Prec<T>& pr, const FullOp<T>& op, bool alloc_all) {
-  (void)alloc_all;
+static void build_prec(Problem& P, Prec<T>& pr, const FullOp<T>& op, const double* ref_xy) {
   Arena& ar = P.ar;
   const bool f64 = std::is_same<T, double>::value;
   build_mg<T>(ar, P.hs, false, P.prm.mg_degree, pr.mgU, P.prm.autotune == 1, P.stream,
@@ -1797,6 +1896,7 @@ static void build_prec(Problem& P, Prec<T>& pr, const FullOp<T>& op, bool alloc_
   pr.sb = ar.alloc<T>(n2); pr.sx = ar.alloc<T>(n2); pr.sx2 = ar.alloc<T>(n2); pr.sd = ar.alloc<T>(n2);
   pr.cs_k = P.prm.cs_degree;
   pr.chs = cheb_coeffs(P.hs.cs_lo, P.hs.cs_hi, pr.cs_k);
+  setup_solid_patches<T>(ar, P.hs, ref_xy, pr);
   const size_t nf = 2 * (size_t)P.nU + 3 * (size_t)P.nP;
   pr.ru = ar.alloc<T>(2 * (size_t)P.nU);
   pr.t = ar.alloc<T>(nf);
@@ -2127,12 +2227,11 @@ static void allocate_problem(Problem& P, const double* ref_xy, const int* tris_h
   P.part = ar.alloc<double>((size_t)std::max(P.red_blocks, 64) * (m + 2));
   P.ctl = ar.alloc<Ctl>(1);
   P.op64 = make_op<double>(P, P.cf_val, P.cft_val);
-  build_prec<double>(P, P.p64, P.op64, true);
+  build_prec<double>(P, P.p64, P.op64, ref_xy);
   if (P.prm.precision == 1) {
     P.op32 = make_op<float>(P, P.cf_val32, P.cft_val32);
-    build_prec<float>(P, P.p32, P.op32, true);
+    build_prec<float>(P, P.p32, P.op32, ref_xy);
   }
-  (void)ref_xy;
 }
 
 

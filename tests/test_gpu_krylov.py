@@ -30,7 +30,7 @@ def _pack(prob, u, p, X, lam):
     (20, 300.0, 0.02, 1e-3, 1, 33),     # several groups, n no multiple of the chunk
     (32, 100.0, 0.1, 1e-3, 1, 2),
     (48, 10.0, 0.1, 1e-2, 1, 2),
-    (208, 10.0, 0.1, 1e-3, 2, 2),       # more than 2^19 unknowns: the larger chunk
+    (224, 10.0, 0.1, 1e-3, 2, 2),       # more than 2^19 unknowns: the larger chunk
 ])
 def test_one_cycle_reaches_its_estimate(N, kappa, nu, dt, stokes_its, least):
     from paper_2301_10041_gb300 import fsi
