@@ -337,8 +337,9 @@ const char* fsi_status_str(int status);
  * cleared: the call returns FSI_ERR_CUDA without launching.  Every call shares
  * the one scratch array and clears the part it uses before using it; calls
  * that overlap on the GPU race on it, so callers must serialise them.  The
- * per-cell lists are sorted by one thread per cell, in time quadratic in the
- * points of a cell (about 50 when the solid mesh size is half the fluid's). */
+ * per-cell lists are sorted by one warp per cell up to 256 points, by one
+ * thread beyond, in time quadratic in the points of a cell (about 50 when the
+ * solid mesh size is half the fluid's). */
 #define FSI_NOALLOC_MAX_CELLS 262144
 int fsi_locate_bin_noalloc(int N, int n_tris, const int* tris, const double* X,
                            int* cell, double* xi, double* eta,

@@ -74,38 +74,48 @@ __global__ void k_na_clear(NoAllocScratch* s, int ncells) {
 }
 
 // same arithmetic as the library's point location: x = P0 + xi1 (P1 - P0) +
-// xi2 (P2 - P0) in explicitly rounded FP64, half-open cells on t = x * N
-__global__ void k_na_locate(int n_pts, int N, const int* __restrict__ tris, const double* __restrict__ X,
-                            int* __restrict__ cell, double* __restrict__ xi, double* __restrict__ eta,
-                            NoAllocScratch* s) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n_pts) return;
-  const int t = p / 6, q = p - 6 * (p / 6);
+// xi2 (P2 - P0) in explicitly rounded FP64, half-open cells on t = x * N.  A
+// thread takes a triangle: the FP64 pipe bounds this kernel (64 cycles a warp
+// instruction), and the six points share the differences of the vertices.  The
+// domain test reads the bits (x in [0, 1] or -0 is one unsigned comparison) and
+// the cell is a truncation, x being non-negative by then.
+__global__ void __launch_bounds__(128) k_na_locate(int n_tris, int N, const int* __restrict__ tris,
+                                                   const double* __restrict__ X, int* __restrict__ cell,
+                                                   double* __restrict__ xi, double* __restrict__ eta,
+                                                   NoAllocScratch* s) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n_tris) return;
   const int v0 = tris[3 * t], v1 = tris[3 * t + 1], v2 = tris[3 * t + 2];
-  const double l1 = c_na_lam[q][1], l2 = c_na_lam[q][2];
-  double loc[2];
-  int idx[2];
-  bool ok = true;
+  double P0[2], d1[2], d2[2];
+#pragma unroll
   for (int c = 0; c < 2; ++c) {
-    const double P0 = X[2 * v0 + c], P1 = X[2 * v1 + c], P2 = X[2 * v2 + c];
-    const double x = __dadd_rn(__dadd_rn(P0, __dmul_rn(l1, __dsub_rn(P1, P0))), __dmul_rn(l2, __dsub_rn(P2, P0)));
-    if (!(x >= 0.0 && x <= 1.0)) { ok = false; idx[c] = 0; loc[c] = 0.0; continue; }
-    const double tc = __dmul_rn(x, (double)N);
-    int i = (int)floor(tc);
-    if (i >= N) i = N - 1;
-    idx[c] = i;
-    loc[c] = __dsub_rn(tc, (double)i);
+    P0[c] = X[2 * v0 + c];
+    d1[c] = __dsub_rn(X[2 * v1 + c], P0[c]);
+    d2[c] = __dsub_rn(X[2 * v2 + c], P0[c]);
   }
-  if (!ok) {
-    cell[p] = -1; xi[p] = 0.0; eta[p] = 0.0;
-    atomicAdd(&s->outside, 1);
-    return;
+  const double fN = (double)N;
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    const double l1 = c_na_lam[q][1], l2 = c_na_lam[q][2];
+    double loc[2];
+    int idx[2];
+    bool ok = true;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const double x = __dadd_rn(__dadd_rn(P0[c], __dmul_rn(l1, d1[c])), __dmul_rn(l2, d2[c]));
+      const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
+      ok = ok && (bits <= 0x3FF0000000000000ull || bits == 0x8000000000000000ull);   // 0 <= x <= 1
+      const double tc = __dmul_rn(x, fN);
+      const int i = min(__double2int_rz(tc), N - 1);
+      idx[c] = i;
+      loc[c] = __dsub_rn(tc, (double)i);
+    }
+    const int p = 6 * t + q, c = idx[1] * N + idx[0];
+    cell[p] = ok ? c : -1;
+    xi[p] = ok ? loc[0] : 0.0;
+    eta[p] = ok ? loc[1] : 0.0;
+    atomicAdd(ok ? &s->count[c] : &s->outside, 1);
   }
-  const int c = idx[1] * N + idx[0];
-  cell[p] = c;
-  xi[p] = loc[0];
-  eta[p] = loc[1];
-  atomicAdd(&s->count[c], 1);
 }
 
 __device__ int na_block_excl_scan(int v, int* sm, int& total) {
@@ -140,24 +150,18 @@ __global__ void k_na_scan_blocks(int n, NoAllocScratch* s) {
   if (threadIdx.x == 0) s->bsum[blockIdx.x] = total;
 }
 
-__global__ void k_na_scan_top(int nb, NoAllocScratch* s) {
-  __shared__ int sm[32];
-  int carry = 0;
-  for (int b0 = 0; b0 < nb; b0 += kNaBlock) {
-    const int i = b0 + threadIdx.x;
-    int total;
-    const int e = na_block_excl_scan(i < nb ? s->bsum[i] : 0, sm, total);
-    if (i < nb) s->bsum[i] = carry + e;
-    carry += total;
-  }
-}
-
+// offsets of a block's cells: the sum of the blocks before it (at most
+// kNaMaxBlocks of them, summed here rather than by a launch of its own) and
+// the scan inside the block
 __global__ void k_na_scan_final(int n, NoAllocScratch* s, int* __restrict__ cell_start) {
   __shared__ int sm[32];
+  static_assert(kNaMaxBlocks <= kNaBlock, "one thread per earlier block");
+  int before;
+  na_block_excl_scan((int)threadIdx.x < (int)blockIdx.x ? s->bsum[threadIdx.x] : 0, sm, before);
   const int i = blockIdx.x * kNaBlock + threadIdx.x;
   const int v = i < n ? s->count[i] : 0;
   int total;
-  const int e = na_block_excl_scan(v, sm, total) + s->bsum[blockIdx.x];
+  const int e = na_block_excl_scan(v, sm, total) + before;
   if (i < n) { cell_start[i] = e; s->cursor[i] = e; }
   if (i == n - 1) cell_start[n] = e + v;
 }
@@ -171,22 +175,45 @@ __global__ void k_na_scatter(int n_pts, const int* __restrict__ cell, int* __res
   cell_points[atomicAdd(&s->cursor[c], 1)] = p;
 }
 
-// the scatter order inside a cell is not fixed: sort each list by point id
-// (insertion sort, one thread per cell: quadratic in the points of one cell,
-// about 50 when the solid mesh size is half the fluid mesh size)
-__global__ void k_na_sort(int ncells, const int* __restrict__ cell_start, int* __restrict__ cell_points) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+// The scatter order inside a cell is not fixed: sort each list by point id.  A
+// warp takes a cell and ranks up to kNaSortMax points by counting the smaller
+// ones (all different) from shared memory; a longer list is sorted in place by
+// one thread.  One thread per cell inserting point by point took 240 of the
+// 293 us of a call with 382 000 points on 256 x 256 cells (some 50 points in
+// each cell the body covers, every step a dependent global read and write); the
+// call takes 57 us now.
+// The first thread also hands over the number of points outside.
+constexpr int kNaSortMax = 256;
+constexpr int kNaSortWarps = 4;
+__global__ void __launch_bounds__(32 * kNaSortWarps) k_na_sort(int ncells, const int* __restrict__ cell_start,
+                                                               int* __restrict__ cell_points,
+                                                               const NoAllocScratch* s, int* __restrict__ n_outside) {
+  __shared__ int list[kNaSortWarps][kNaSortMax];
+  if (blockIdx.x == 0 && threadIdx.x == 0) *n_outside = s->outside;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int c = blockIdx.x * kNaSortWarps + w;
   if (c >= ncells) return;
-  const int a = cell_start[c], b = cell_start[c + 1];
-  for (int i = a + 1; i < b; ++i) {
+  const int a = cell_start[c], n = cell_start[c + 1] - a;
+  if (n <= 1) return;
+  if (n <= kNaSortMax) {
+    for (int i = lane; i < n; i += 32) list[w][i] = cell_points[a + i];
+    __syncwarp();
+    for (int i = lane; i < n; i += 32) {
+      const int v = list[w][i];
+      int r = 0;
+      for (int k = 0; k < n; ++k) r += list[w][k] < v;
+      cell_points[a + r] = v;
+    }
+    return;
+  }
+  if (lane != 0) return;
+  for (int i = a + 1; i < a + n; ++i) {
     const int v = cell_points[i];
     int j = i - 1;
     while (j >= a && cell_points[j] > v) { cell_points[j + 1] = cell_points[j]; --j; }
     cell_points[j + 1] = v;
   }
 }
-
-__global__ void k_na_outside(const NoAllocScratch* s, int* out) { *out = s->outside; }
 
 unsigned nb(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
@@ -238,13 +265,11 @@ int run_locate_bin(int dev, int N, int n_tris, const int* tris, const double* X,
   const int nc = (int)ncells;
   const unsigned nblocks = nb(nc, kNaBlock);
   k_na_clear<<<nb(nc, 256), 256, 0, stream>>>(s, nc);
-  k_na_locate<<<nb(n_pts, 256), 256, 0, stream>>>(n_pts, N, tris, X, cell, xi, eta, s);
+  k_na_locate<<<nb(n_tris, 128), 128, 0, stream>>>(n_tris, N, tris, X, cell, xi, eta, s);
   k_na_scan_blocks<<<nblocks, kNaBlock, 0, stream>>>(nc, s);
-  k_na_scan_top<<<1, kNaBlock, 0, stream>>>((int)nblocks, s);
   k_na_scan_final<<<nblocks, kNaBlock, 0, stream>>>(nc, s, cell_start);
   k_na_scatter<<<nb(n_pts, 256), 256, 0, stream>>>(n_pts, cell, cell_points, s);
-  k_na_sort<<<nb(nc, 128), 128, 0, stream>>>(nc, cell_start, cell_points);
-  k_na_outside<<<1, 1, 0, stream>>>(s, n_outside);
+  k_na_sort<<<nb(nc, kNaSortWarps), 32 * kNaSortWarps, 0, stream>>>(nc, cell_start, cell_points, s, n_outside);
   if (cudaGetLastError() != cudaSuccess) return FSI_ERR_CUDA;
   return FSI_OK;
 }
