@@ -1782,6 +1782,29 @@ __global__ void __launch_bounds__(256) k_xupdate(int n2, double* __restrict__ x,
   reinterpret_cast<double2*>(x)[i] = v;
 }
 
+// nodal velocities on the lattice -> node order, as u^n and as the iterate
+__global__ void k_state_in(size_t nlat, const int* __restrict__ l2n, const double* __restrict__ u,
+                           double* __restrict__ uold, double* __restrict__ x) {
+  pdl_begin();
+  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (i >= nlat) return;
+  const int k = l2n[i];
+  if (k < 0) return;   // the walls keep their data
+  const double2 v = reinterpret_cast<const double2*>(u)[i];
+  reinterpret_cast<double2*>(uold)[k] = v;
+  reinterpret_cast<double2*>(x)[k] = v;
+}
+
+// node order -> lattice, wall values included
+__global__ void k_state_out(size_t nlat, const int* __restrict__ l2n, const double* __restrict__ wall,
+                            const double* __restrict__ x, double* __restrict__ u) {
+  pdl_begin();
+  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (i >= nlat) return;
+  const int k = l2n[i];
+  reinterpret_cast<double2*>(u)[i] = k >= 0 ? reinterpret_cast<const double2*>(x)[k] : reinterpret_cast<const double2*>(wall)[i];
+}
+
 // zero mean of the constant pressure coefficients (p in L^2_0)
 __global__ void __launch_bounds__(kRedThreads) k_pmean(int nP, double* __restrict__ p, double* __restrict__ part,
                                                        Ctl* ctl) {
@@ -2280,25 +2303,23 @@ static int map_exception() {
   }
 }
 
+// State in and out.  The caller's nodal arrays cross in one copy each, to and
+// from a scratch area on the device (the Krylov basis, idle between solves: it
+// holds at least two vectors of n, more than the lattice's 2 (2N+1)^2 for every
+// N >= 2), and two kernels permute between lattice and node order there.  On the
+// host the same took an index loop over the nodes, a second upload and, on the
+// way out, a zeroed copy of the whole vector.
 static void upload_state(Problem& P, const double* u, const double* X) {
-  const int n1 = 2 * P.N + 1;
+  const size_t nlat = (size_t)(2 * P.N + 1) * (2 * P.N + 1);
   if (u) {
-    std::vector<double> ui(2 * (size_t)P.nU);
-    for (int k = 0; k < P.nU; ++k) {
-      const int lat = P.hs.interior_lattice[k];
-      ui[2 * k] = u[2 * (size_t)lat];
-      ui[2 * k + 1] = u[2 * (size_t)lat + 1];
-    }
-    CK(cudaMemcpyAsync(P.uold, ui.data(), ui.size() * 8, cudaMemcpyHostToDevice, P.stream));
-    CK(cudaMemcpyAsync(P.x, ui.data(), ui.size() * 8, cudaMemcpyHostToDevice, P.stream));
-    CK(cudaStreamSynchronize(P.stream));
+    CK(cudaMemcpyAsync(P.V, u, 2 * nlat * 8, cudaMemcpyHostToDevice, P.stream));
+    launch(k_state_in, nblk(nlat, 256), 256, 0, P.stream, nlat, P.l2n, (const double*)P.V, P.uold, P.x);
   }
   if (X) {
     CK(cudaMemcpyAsync(P.Xold, X, 2 * (size_t)P.nS * 8, cudaMemcpyHostToDevice, P.stream));
-    CK(cudaMemcpyAsync(P.x + P.offX, X, 2 * (size_t)P.nS * 8, cudaMemcpyHostToDevice, P.stream));
-    CK(cudaStreamSynchronize(P.stream));
+    CK(cudaMemcpyAsync(P.x + P.offX, P.Xold, 2 * (size_t)P.nS * 8, cudaMemcpyDeviceToDevice, P.stream));
   }
-  (void)n1;
+  if (u || X) CK(cudaStreamSynchronize(P.stream));
 }
 
 static size_t footprint_impl(const fsi_params& prm0, int n_nodes, int n_tris, const double* ref_xy,
@@ -2714,21 +2735,15 @@ int fsi_get_state(fsi_problem* h, double* u, double* pr, double* X, double* lam)
   if (!h) return FSI_ERR_INVALID;
   Problem& P = h->P;
   try {
-    std::vector<double> x(P.n);
-    CK(cudaMemcpyAsync(x.data(), P.x, P.n * 8, cudaMemcpyDeviceToHost, P.stream));
-    CK(cudaStreamSynchronize(P.stream));
+    const size_t nlat = (size_t)(2 * P.N + 1) * (2 * P.N + 1);
     if (u) {
-      const size_t nl = (size_t)(2 * P.N + 1) * (2 * P.N + 1);
-      std::copy(P.hs.wall_u.begin(), P.hs.wall_u.begin() + 2 * nl, u);
-      for (int k = 0; k < P.nU; ++k) {
-        const int lat = P.hs.interior_lattice[k];
-        u[2 * (size_t)lat] = x[2 * (size_t)k];
-        u[2 * (size_t)lat + 1] = x[2 * (size_t)k + 1];
-      }
+      launch(k_state_out, nblk(nlat, 256), 256, 0, P.stream, nlat, P.l2n, P.wall, (const double*)P.x, P.V);
+      CK(cudaMemcpyAsync(u, P.V, 2 * nlat * 8, cudaMemcpyDeviceToHost, P.stream));
     }
-    if (pr) std::copy(x.begin() + P.offP, x.begin() + P.offX, pr);
-    if (X) std::copy(x.begin() + P.offX, x.begin() + P.offL, X);
-    if (lam) std::copy(x.begin() + P.offL, x.end(), lam);
+    if (pr) CK(cudaMemcpyAsync(pr, P.x + P.offP, 3 * (size_t)P.nP * 8, cudaMemcpyDeviceToHost, P.stream));
+    if (X) CK(cudaMemcpyAsync(X, P.x + P.offX, 2 * (size_t)P.nS * 8, cudaMemcpyDeviceToHost, P.stream));
+    if (lam) CK(cudaMemcpyAsync(lam, P.x + P.offL, 2 * (size_t)P.nS * 8, cudaMemcpyDeviceToHost, P.stream));
+    CK(cudaStreamSynchronize(P.stream));
     return FSI_OK;
   } catch (...) {
     return map_exception();
