@@ -98,9 +98,9 @@ typedef struct fsi_params {
     int    mg_cluster; /* 0: automatic -- the coarse multigrid levels whose operators
                           fit in the shared memory of one thread-block cluster
                           run as one cluster launch per V-cycle (same
-                          arithmetic), except that an FP32 hierarchy with the
-                          fused matrix-free levels (mg_fused = 0) keeps only
-                          levels of at most 8 cells there; -1: no cluster; n > 0:
+                          arithmetic), except that with the matrix-free levels
+                          (mg_fused = 0) only levels of at most 8 cells stay
+                          there; -1: no cluster; n > 0:
                           levels of at most n cells a side in the cluster */
     int    coupling;   /* C_f(X^n) quadrature: 0 = the degree-4 6-point rule at
                           points located in the fluid grid; 1 = exact, by
@@ -129,11 +129,12 @@ typedef struct fsi_params {
                           with A_s, C_s and the C_f point rule by the 3 x 3
                           Gauss rule on each element.  Q1 takes coupling 0 and
                           solid_law 0 only */
-    int    mg_fused;   /* 0: the finest multigrid levels of the FP32 hierarchy
-                          (down to the cluster-resident ones, at least 16 cells a
-                          side) run matrix-free, each V-cycle level as two fused
+    int    mg_fused;   /* 0: the multigrid levels run matrix-free: the finest levels
+                          of the FP32 hierarchy (down to the cluster-resident ones,
+                          at least 16 cells a side) each as two fused
                           launches (pre-smoothing + residual + restriction;
-                          prolongation + post-smoothing); -1: the per-level
+                          prolongation + post-smoothing), the FP64 levels of 32
+                          cells or more product by product; -1: the per-level
                           sparse kernels on every level */
     int    mg_coarse;  /* the coarsening stops at the first grid of at most
                           mg_coarse cells a side, whose operators are inverted

@@ -17,7 +17,8 @@ LIB = os.path.join(OUT_DIR, "libfsi_gb300.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["fsi_solver.cu", "fsi_setup.cpp", "fsi_noalloc.cu"]
 HEADERS = ["fsi_internal.h", "fsi_kernels.cuh", "fsi_coupling.cuh", "fsi_cluster.cuh", "fsi_cluster_host.h", "fsi_solid.cuh",
-           "fsi_mgfused.cuh", "fsi_solid_cheb.cuh"]
+           "fsi_mgfused.cuh", "fsi_solid_cheb.cuh",
+           "fsi_mfop.cuh"]
 
 
 def nvcc() -> str:

@@ -352,6 +352,60 @@ struct FullOp {
   const TA* kt = nullptr;             // nonlinear solid: 2x2 tangent blocks in the Ssol slots
 };
 
+// The solid rows of the full operator: CTA b of 128 threads takes 32 nodes, four
+// threads each.
+template <class TA, class TX, class TY>
+__device__ __forceinline__ void fullmv_solid_rows(const FullOp<TA>& op, int b, const TX* __restrict__ x,
+                                                  TY* __restrict__ y, const TY* __restrict__ z, TY alpha, TY beta) {
+  const int lane = threadIdx.x & 31, t = lane >> 3;
+  const int wrow = (threadIdx.x >> 5) * kSliceRows + (lane & 7);
+  const size_t offP = 2 * (size_t)op.nU, offX = offP + 3 * (size_t)op.nP, offL = offX + 2 * (size_t)op.nS;
+  const int r = b * 32 + wrow;
+  const bool live = r < op.nS;
+  TA a[4] = {0, 0, 0, 0};
+  if (live) {
+    const int base = op.Ssol.soff[r >> 3] + (r & 7), n = op.Ssol.len[r];
+    for (int k = t; k < n; k += kRowThreads) {
+      const int slot = base + (k << 3);
+      const int c = __ldg(op.Ssol.col + slot);
+      const TA as = __ldg(op.Ssol.val + 2 * (size_t)slot), cs = __ldg(op.Ssol.val + 2 * (size_t)slot + 1);
+      TA Xv[2], Lv[2];
+      load_x<TX, TA, 2>(x + offX, c, Xv);
+      load_x<TX, TA, 2>(x + offL, c, Lv);
+      if (op.kt) {  // tangent of the nonlinear law: a 2x2 block per slot
+        const TA* kb = op.kt + 4 * (size_t)slot;
+        a[0] += kb[0] * Xv[0] + kb[1] * Xv[1] - cs * Lv[0];
+        a[1] += kb[2] * Xv[0] + kb[3] * Xv[1] - cs * Lv[1];
+      } else {
+        a[0] += as * Xv[0] - cs * Lv[0];
+        a[1] += as * Xv[1] - cs * Lv[1];
+      }
+      a[2] -= op.inv_dt * cs * Xv[0];
+      a[3] -= op.inv_dt * cs * Xv[1];
+    }
+    const size_t cbase = (size_t)(r >> 5) * 32 * op.cf_cap + (r & 31);
+    const int nc = op.cf_len[r];
+    for (int k = t; k < nc; k += kRowThreads) {
+      const size_t slot = cbase + ((size_t)k << 5);
+      const int c = op.cf_col[slot];
+      const TA v = op.cf_val[slot];
+      TA uv[2];
+      load_x<TX, TA, 2>(x, c, uv);
+      a[2] += v * uv[0];
+      a[3] += v * uv[1];
+    }
+  }
+  row_reduce<TA, 4>(a);
+  if (!live || t != 0) return;
+  TY o[4] = {alpha * (TY)a[0], alpha * (TY)a[1], alpha * (TY)a[2], alpha * (TY)a[3]};
+  if (z) {
+    o[0] += beta * z[offX + 2 * r]; o[1] += beta * z[offX + 2 * r + 1];
+    o[2] += beta * z[offL + 2 * r]; o[3] += beta * z[offL + 2 * r + 1];
+  }
+  y[offX + 2 * r] = o[0]; y[offX + 2 * r + 1] = o[1];
+  y[offL + 2 * r] = o[2]; y[offL + 2 * r + 1] = o[3];
+}
+
 template <class TA, class TX, class TY>
 __global__ void __launch_bounds__(128, sizeof(TA) == 4 ? 16 : 8) k_fullmv(FullOp<TA> op, const TX* __restrict__ x, TY* __restrict__ y,
                                                 const TY* __restrict__ z, TY alpha, TY beta,
@@ -412,50 +466,7 @@ __global__ void __launch_bounds__(128, sizeof(TA) == 4 ? 16 : 8) k_fullmv(FullOp
       y[offP + 3 * r + i] = o;
     }
   } else {
-    const int r = (b - op.gU - op.gP) * 32 + wrow;
-    const bool live = r < op.nS;
-    TA a[4] = {0, 0, 0, 0};
-    if (live) {
-      const int base = op.Ssol.soff[r >> 3] + (r & 7), n = op.Ssol.len[r];
-      for (int k = t; k < n; k += kRowThreads) {
-        const int slot = base + (k << 3);
-        const int c = __ldg(op.Ssol.col + slot);
-        const TA as = __ldg(op.Ssol.val + 2 * (size_t)slot), cs = __ldg(op.Ssol.val + 2 * (size_t)slot + 1);
-        TA Xv[2], Lv[2];
-        load_x<TX, TA, 2>(x + offX, c, Xv);
-        load_x<TX, TA, 2>(x + offL, c, Lv);
-        if (op.kt) {  // tangent of the nonlinear law: a 2x2 block per slot
-          const TA* kb = op.kt + 4 * (size_t)slot;
-          a[0] += kb[0] * Xv[0] + kb[1] * Xv[1] - cs * Lv[0];
-          a[1] += kb[2] * Xv[0] + kb[3] * Xv[1] - cs * Lv[1];
-        } else {
-          a[0] += as * Xv[0] - cs * Lv[0];
-          a[1] += as * Xv[1] - cs * Lv[1];
-        }
-        a[2] -= op.inv_dt * cs * Xv[0];
-        a[3] -= op.inv_dt * cs * Xv[1];
-      }
-      const size_t cbase = (size_t)(r >> 5) * 32 * op.cf_cap + (r & 31);
-      const int nc = op.cf_len[r];
-      for (int k = t; k < nc; k += kRowThreads) {
-        const size_t slot = cbase + ((size_t)k << 5);
-        const int c = op.cf_col[slot];
-        const TA v = op.cf_val[slot];
-        TA uv[2];
-        load_x<TX, TA, 2>(x, c, uv);
-        a[2] += v * uv[0];
-        a[3] += v * uv[1];
-      }
-    }
-    row_reduce<TA, 4>(a);
-    if (!live || t != 0) return;
-    TY o[4] = {alpha * (TY)a[0], alpha * (TY)a[1], alpha * (TY)a[2], alpha * (TY)a[3]};
-    if (z) {
-      o[0] += beta * z[offX + 2 * r]; o[1] += beta * z[offX + 2 * r + 1];
-      o[2] += beta * z[offL + 2 * r]; o[3] += beta * z[offL + 2 * r + 1];
-    }
-    y[offX + 2 * r] = o[0]; y[offX + 2 * r + 1] = o[1];
-    y[offL + 2 * r] = o[2]; y[offL + 2 * r + 1] = o[3];
+    fullmv_solid_rows<TA, TX, TY>(op, b - op.gU - op.gP, x, y, z, alpha, beta);
   }
 }
 

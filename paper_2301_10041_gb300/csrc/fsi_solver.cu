@@ -32,6 +32,7 @@
 #include "fsi_internal.h"
 #include "fsi_kernels.cuh"
 #include "fsi_mgfused.cuh"
+#include "fsi_mfop.cuh"
 #include "fsi_solid.cuh"
 #include "fsi_solid_cheb.cuh"
 
@@ -314,6 +315,8 @@ struct MGLevel {
   bool mf = false;
   MfVelOp<T> mfu;        // velocity hierarchy
   T* mftab = nullptr;    // pressure hierarchy: kMfPresTab values
+  MfOp<T> mfo;           // velocity hierarchy: the level's product matrix-free (mfo.N > 0)
+  bool mfl = false;      // pressure hierarchy: the same, from mftab
   T divB[3][9][2] = {};  // entries of -B and -B^T on this level (residual start)
 };
 
@@ -399,8 +402,62 @@ static void build_coarse_inverse(Arena& ar, const HostSetup& hs, bool pressure, 
   }
 }
 
+// The level's velocity stencils as MfOp; none (N = 0) when the grid has none or
+// a block is not of the form the kernels use: equal off-diagonal entries, zero
+// for two nodes on one grid line.
 template <class T>
-static void build_mg(Arena& ar, const HostSetup& hs, bool pressure, int degree, MG<T>& mg, bool tune,
+static MfOp<T> make_mfop(const FluidLevelHost& H) {
+  MfOp<T> m;
+  if (!H.mf) return m;
+  for (int t = 0; t < 4; ++t)
+    for (int y = 0; y < 5; ++y)
+      for (int x = 0; x < 5; ++x) {
+        const double* c = H.stenA[t][y][x];
+        if (c[1] != c[2] || ((x == 2 || y == 2) && c[1] != 0.0)) return m;
+        m.c[t][y][x][0] = (T)c[0];
+        m.c[t][y][x][1] = (T)c[1];
+        m.c[t][y][x][2] = (T)c[3];
+      }
+  for (int k = 0; k < 3; ++k)
+    for (int q = 0; q < 9; ++q)
+      for (int d = 0; d < 2; ++d) m.divB[k][q][d] = (T)H.divB[k][q][d];
+  m.N = H.N;
+  return m;
+}
+
+// Smallest grids of the FP64 matrix-free products: below, a row's serial chain of
+// FP64 multiply-adds is longer than the sparse kernels' (which split it four
+// ways).  One smoothing step, sparse against matrix-free: velocity 20.3 -> 10.0 us
+// on 128 cells, 7.4 -> 4.8 on 64, 4.7 -> 4.4 on 32; pressure 9.9 -> 4.6 on 128,
+// 5.2 -> 3.3 on 64.  Full operator 33.9 -> 19.2 on 128 cells, but 7.2 against
+// 10.3 us on 16.
+constexpr int kMfo64MinN = 32;       // velocity and pressure levels
+constexpr int kMfo64MinNFull = 64;   // full operator and Stokes residual
+
+// One product of a level with the epilogue of a.mode: matrix-free where the
+// level says so, else the sliced-ELL kernel.
+template <class T>
+static void level_launch(const MGLevel<T>& L, int mode, const SpmvArgs<T>& a, cudaStream_t s) {
+  if (L.mfo.N > 0) {
+    const unsigned g = mfop_grid<T>(L.mfo.N);
+    if (mode == MODE_AXPBY) launch(k_mfv<T, MODE_AXPBY>, g, 128, 0, s, L.mfo, a);
+    else if (mode == MODE_CHEB) launch(k_mfv<T, MODE_CHEB>, g, 128, 0, s, L.mfo, a);
+    else if (mode == MODE_CHEB0) launch(k_mfv<T, MODE_CHEB0>, g, 128, 0, s, L.mfo, a);
+    else throw std::logic_error("level_launch");
+    return;
+  }
+  if (L.mfl) {
+    const unsigned g = nblk(3 * (size_t)L.N * L.N, 96);
+    if (mode == MODE_CHEB) launch(k_mfp<T, MODE_CHEB>, g, 96, 0, s, L.N, (const T*)L.mftab, a);
+    else if (mode == MODE_CHEB0) launch(k_mfp<T, MODE_CHEB0>, g, 96, 0, s, L.N, (const T*)L.mftab, a);
+    else throw std::logic_error("level_launch");
+    return;
+  }
+  sell_launch(L.A, mode, a, s);
+}
+
+template <class T>
+static void build_mg(Arena& ar, const HostSetup& hs, bool pressure, int degree, MG<T>& mg, bool tune, bool mfree,
                      cudaStream_t s, const double* inv64 = nullptr, int ld64 = 0) {
   const int nl = pressure ? hs.nlev_p : hs.nlev_u;
   mg.degree = degree;
@@ -448,7 +505,9 @@ static void build_mg(Arena& ar, const HostSetup& hs, bool pressure, int degree, 
       for (int v = 0; v < 9; ++v)
         for (int k = 0; k < 3; ++k) tab[kMfPresDinv + 3 * v + k] = H.dinvLv[v][k];
       L.mftab = upload_as<T>(ar, tab);
+      L.mfl = mfree && H.N >= kMfo64MinN;
     }
+    if (mfree && !pressure && H.N >= kMfo64MinN) L.mfo = make_mfop<T>(H);
   }
   build_coarse_inverse<T>(ar, hs, pressure, mg, inv64, ld64, s);
 }
@@ -782,12 +841,12 @@ static T* vcycle(MG<T>& mg, int l, cudaStream_t s, T* out, const SpmvArgs<T>* fi
     SpmvArgs<T> a;
     a.x = xc; a.y = xn; a.z = L.b; a.d = L.d; a.dinv = L.dinv;
     a.c1 = (T)L.ch.c1[i - 1]; a.c2 = (T)L.ch.c2[i - 1];
-    sell_launch(L.A, MODE_CHEB, a, s);
+    level_launch(L, MODE_CHEB, a, s);
     std::swap(xc, xn);
   }
   MGLevel<T>& C = mg.lv[l + 1];
   if (L.RA.nrows == 0) {  // residual, then its restriction
-    sell_launch(L.A, MODE_AXPBY, axpby<T>(xc, L.r, L.b, (T)-1, (T)1), s);
+    level_launch(L, MODE_AXPBY, axpby<T>(xc, L.r, L.b, (T)-1, (T)1), s);
     if (l + 1 == last || (mg.cl.on && l + 1 == mg.cl.lc)) {
       sell_launch(L.R, MODE_AXPBY, axpby<T>(L.r, C.b, nullptr, (T)1, (T)0), s);
     } else {
@@ -816,8 +875,8 @@ static T* vcycle(MG<T>& mg, int l, cudaStream_t s, T* out, const SpmvArgs<T>* fi
       if (fused) *fused = true;
     }
     a.x = xc; a.y = dst; a.z = L.b; a.d = L.d; a.dinv = L.dinv;
-    if (i == 0) { a.c2 = (T)L.ch.c0; sell_launch(L.A, MODE_CHEB0, a, s); }
-    else { a.c1 = (T)L.ch.c1[i - 1]; a.c2 = (T)L.ch.c2[i - 1]; sell_launch(L.A, MODE_CHEB, a, s); }
+    if (i == 0) { a.c2 = (T)L.ch.c0; level_launch(L, MODE_CHEB0, a, s); }
+    else { a.c1 = (T)L.ch.c1[i - 1]; a.c2 = (T)L.ch.c2[i - 1]; level_launch(L, MODE_CHEB, a, s); }
     if (dst == out) return out;
     std::swap(xc, xn);
   }
@@ -829,6 +888,7 @@ template <class T>
 struct Prec {
   MG<T> mgU, mgP;
   FullOp<T> op;          // operator in this precision (shares structure arrays)
+  MfOp<T> mf;            // its fluid rows matrix-free (mf.N > 0)
   Sell<T> Cs, As;
   T* mpinv = nullptr;    // inverse P1disc mass diagonal
   T* csdinv = nullptr;   // inverse diagonal of the solid mass
@@ -1132,7 +1192,10 @@ static void stokes_velocity(Problem& P, Prec<T>& pr, const T* in_u, const T* p, 
     return;
   }
   if (zu) throw std::logic_error("stokes_velocity: the residual start needs the fused finest level");
-  if (p) {
+  if (p && L0u.mfo.N > 0) {
+    launch(k_mfv_start<T>, mfop_grid<T>(L0u.mfo.N), 128, 0, s, L0u.mfo, in_u, p, (const T*)L0u.dinv,
+           (T)L0u.ch.c0, L0u.b, L0u.d, L0u.x);
+  } else if (p) {
     SpmvArgs<T> a;
     a.x = p; a.y = L0u.b; a.z = in_u; a.alpha = -1; a.beta = 1;
     a.d = L0u.d; a.dinv = L0u.dinv; a.xo = L0u.x; a.c2 = (T)L0u.ch.c0;
@@ -1168,6 +1231,37 @@ static void stokes_apply(Problem& P, Prec<T>& pr, const T* in_u, const T* in_p, 
   } else {
     stokes_pressure(P, pr, in_p, out_p, s);
     stokes_velocity(P, pr, in_u, (const T*)out_p, out_u, s);
+  }
+}
+
+// Residual of the Stokes block at pr.zw for the right-hand side (vu, vp) into
+// pr.t; with start, the pressure rows also start their V-cycle.
+template <class T>
+static void stokes_res_launch(Problem& P, Prec<T>& pr, const T* vu, const T* vp, bool start, cudaStream_t s) {
+  MGLevel<T>& L = pr.mgP.lv[0];
+  const T* dinv = start ? L.dinv : nullptr;
+  T *b = start ? L.b : nullptr, *d = start ? L.d : nullptr, *x = start ? L.x : nullptr;
+  if (pr.mf.N > 0) {
+    const unsigned gU = mfop_grid<T>(pr.mf.N);
+    launch(k_mf_stokes_res<T>, gU + nblk((size_t)P.nP * (3 / mfop_prows<T>()), 128), 128, 0, s, pr.mf, (int)gU, P.nU, P.nP, pr.zw, vu, vp, pr.t, dinv,
+           (T)L.ch.c0, b, d, x);
+  } else {
+    launch(k_stokes_res<T>, pr.op.gU + pr.op.gP, 128, 0, s, pr.op, pr.zw, vu, vp, pr.t, dinv, (T)L.ch.c0, b, d, x);
+  }
+}
+
+// y = alpha A x + beta z for the full operator; with Z, x is also stored as its
+// column ctl->j.
+template <class T, class TY>
+static void full_launch(const Prec<T>& pr, const T* x, TY* y, const TY* z, TY alpha, TY beta, T* Z, size_t zld,
+                        const Ctl* ctl, cudaStream_t s) {
+  const FullOp<T>& op = pr.op;
+  if (pr.mf.N > 0) {
+    const unsigned gU = mfop_grid<T>(pr.mf.N), gP = nblk((size_t)op.nP * (3 / mfop_prows<T>()), 128);
+    launch(k_fullmv_mf<T, TY>, gU + gP + op.gS, 128, 0, s, op, pr.mf, (int)gU, (int)gP, x, y, z, alpha, beta, Z, zld,
+           ctl);
+  } else {
+    launch(k_fullmv<T, T, TY>, op.gU + op.gP + op.gS, 128, 0, s, op, x, y, z, alpha, beta, Z, zld, ctl);
   }
 }
 
@@ -1217,8 +1311,7 @@ static void precond_launch(Problem& P, Prec<T>& pr, cudaStream_t s) {
   MGLevel<T>& L0p = pr.mgP.lv[0];
   for (int it = 1; it < pr.stokes_its; ++it) {
     if (split) {
-      launch(k_stokes_res<T>, pr.op.gU + pr.op.gP, 128, 0, s, pr.op, pr.zw, vu, vp, pr.t, (const T*)nullptr, (T)0,
-             (T*)nullptr, (T*)nullptr, (T*)nullptr);
+      stokes_res_launch<T>(P, pr, vu, vp, false, s);
       stokes_apply(P, pr, pr.t, pr.t + P.offP, pr.dz, pr.dz + P.offP, s, split);
       launch(k_axpy<T>, nblk(nf, 256), 256, 0, s, nf, pr.stokes_omega, pr.dz, pr.zw);
     } else if (L0p.mf && pr.mgU.lv[0].mf && (double)pr.stokes_omega == 1.0) {
@@ -1232,12 +1325,7 @@ static void precond_launch(Problem& P, Prec<T>& pr, cudaStream_t s) {
     } else {
       // residual (starting the pressure smoother), then the pressure and
       // velocity corrections, each added to z by its own last kernel
-      if (L0p.mf)
-        launch(k_stokes_res<T>, pr.op.gU + pr.op.gP, 128, 0, s, pr.op, pr.zw, vu, vp, pr.t, (const T*)nullptr, (T)0,
-               (T*)nullptr, (T*)nullptr, (T*)nullptr);
-      else
-        launch(k_stokes_res<T>, pr.op.gU + pr.op.gP, 128, 0, s, pr.op, pr.zw, vu, vp, pr.t, (const T*)L0p.dinv,
-               (T)L0p.ch.c0, L0p.b, L0p.d, L0p.x);
+      stokes_res_launch<T>(P, pr, vu, vp, !L0p.mf, s);
       stokes_pressure(P, pr, pr.t + P.offP, pr.dz + P.offP, s, true, pr.zw + P.offP, pr.stokes_omega);
       stokes_velocity(P, pr, pr.t, (const T*)(pr.dz + P.offP), pr.dz, s, pr.zw, pr.stokes_omega);
     }
@@ -1886,16 +1974,20 @@ template <class T>
 static void build_prec(Problem& P, Prec<T>& pr, const FullOp<T>& op, const double* ref_xy) {
   Arena& ar = P.ar;
   const bool f64 = std::is_same<T, double>::value;
-  build_mg<T>(ar, P.hs, false, P.prm.mg_degree, pr.mgU, P.prm.autotune == 1, P.stream,
+  // the FP64 levels are matrix-free products launch by launch (the FP32 ones
+  // take the fused kernels); mg_fused = -1 keeps the stored matrices
+  const bool mfree = f64 && P.prm.mg_fused == 0;
+  build_mg<T>(ar, P.hs, false, P.prm.mg_degree, pr.mgU, P.prm.autotune == 1, mfree, P.stream,
               f64 ? nullptr : P.p64.mgU.coarse_inv, P.p64.mgU.coarse_ld);
-  build_mg<T>(ar, P.hs, true, P.prm.mg_degree, pr.mgP, P.prm.autotune == 1, P.stream,
+  build_mg<T>(ar, P.hs, true, P.prm.mg_degree, pr.mgP, P.prm.autotune == 1, mfree, P.stream,
               f64 ? nullptr : P.p64.mgP.coarse_inv, P.p64.mgP.coarse_ld);
-  // With the fused matrix-free levels (FP32, every level of 16 cells or more)
-  // the automatic choice leaves the cluster out: two fused launches per level
-  // measured faster than the cluster launch of the same levels on GB300
-  // (10.8 against 9.7 steps/s on the 128 x 128 cavity).
+  // With the matrix-free levels the automatic choice leaves the cluster out:
+  // two fused launches per level measured faster than the cluster launch of
+  // the same levels in FP32 (10.8 against 9.7 steps/s on the 128 x 128
+  // cavity), and in FP64 the pressure cluster from 32 cells down takes 42 us
+  // where its levels launch by launch take 20.
   int cl_max = P.prm.mg_cluster;
-  if (cl_max == 0 && std::is_same<T, float>::value && P.prm.mg_fused == 0) cl_max = 8;
+  if (cl_max == 0 && P.prm.mg_fused == 0) cl_max = 8;
   if (cl_max >= 0) {
     setup_cluster<T>(ar, P.hs, pr.mgU, false, cl_max);
     setup_cluster<T>(ar, P.hs, pr.mgP, true, cl_max);
@@ -1903,6 +1995,7 @@ static void build_prec(Problem& P, Prec<T>& pr, const FullOp<T>& op, const doubl
   select_mf<T>(pr.mgU, P.hs, P.prm.mg_fused, ar.count_only);
   select_mf<T>(pr.mgP, P.hs, P.prm.mg_fused, ar.count_only);
   pr.op = op;
+  if (!f64 || P.N >= kMfo64MinNFull) pr.mf = make_mfop<T>(P.hs.levels[0]);
   pr.Cs = upload_sell<T>(ar, to_sell(P.hs.Cs));
   pr.As = upload_sell<T>(ar, to_sell(P.hs.As));
   if (P.prm.solid_law == 1) {
@@ -2016,16 +2109,14 @@ static void orthogonalise_launch(Problem& P, Prec<T>& pr, const KrylovArgs& k, c
 template <class T>
 static void iteration_launch(Problem& P, Prec<T>& pr, const KrylovArgs& k, cudaStream_t s) {
   precond_launch(P, pr, s);
-  launch(k_fullmv<T, T, double>, pr.op.gU + pr.op.gP + pr.op.gS, 128, 0, s, pr.op, pr.zw, P.w, nullptr, 1.0, 0.0,
-         (T*)P.Z, P.n, (const Ctl*)P.ctl);
+  full_launch<T, double>(pr, pr.zw, P.w, nullptr, 1.0, 0.0, (T*)P.Z, P.n, P.ctl, s);
   if (k.chunk == kChunkSmall) orthogonalise_launch<kChunkSmall>(P, pr, k, s);
   else orthogonalise_launch<kChunkLarge>(P, pr, k, s);
 }
 
 template <class T>
 static void cycle_start_launch(Problem& P, Prec<T>& pr, const KrylovArgs& k, cudaStream_t s) {
-  launch(k_fullmv<double, double, double>, P.op64.gU + P.op64.gP + P.op64.gS, 128, 0, s, P.op64, P.x, P.w, P.b, -1.0,
-         1.0, (double*)nullptr, (size_t)0, (const Ctl*)nullptr);
+  full_launch<double, double>(P.p64, P.x, P.w, P.b, -1.0, 1.0, nullptr, 0, nullptr, s);
   launch(k_cycle_start, P.red_blocks, kRedThreads, 0, s, k);
   launch(k_basis<T>, nblk(P.n / 2, 256), 256, 0, s, (int)(P.n / 2), P.V, P.n, P.w, pr.vin, P.ctl);
 }
@@ -2265,9 +2356,10 @@ static double sell_bytes(const HostBlockMatrix& A) {
 }
 
 template <class T>
-static double fullop_bytes(Problem& P, double cfnnz, size_t xbytes, size_t ybytes) {
+static double fullop_bytes(Problem& P, bool mf, double cfnnz, size_t xbytes, size_t ybytes) {
   const HostSetup& hs = P.hs;
-  double b = sell_bytes<T>(hs.levels[0].A) + sell_bytes<T>(hs.Bt) + sell_bytes<T>(hs.Bneg) + sell_bytes<T>(hs.Ssol);
+  double b = sell_bytes<T>(hs.Ssol);   // matrix-free fluid rows read no stored blocks
+  if (!mf) b += sell_bytes<T>(hs.levels[0].A) + sell_bytes<T>(hs.Bt) + sell_bytes<T>(hs.Bneg);
   b += 2.0 * cfnnz * (sizeof(T) + sizeof(int)) + (P.nU + 1) * 4.0 + P.nS * 4.0;
   b += (double)P.n * (xbytes + ybytes);
   return b;
@@ -2825,11 +2917,9 @@ int fsi_apply_operator(fsi_problem* h, const double* xh, double* yh, int precisi
     CK(cudaMemcpyAsync(tmp, xh, P.n * 8, cudaMemcpyHostToDevice, P.stream));
     if (precision == 1) {
       launch(k_convert<double, float>, nblk(P.n, 256), 256, 0, P.stream, P.n, tmp, P.p32.vin);
-      launch(k_fullmv<float, float, double>, P.op32.gU + P.op32.gP + P.op32.gS, 128, 0, P.stream, P.op32, P.p32.vin, P.w,
-             nullptr, 1.0, 0.0, (float*)nullptr, (size_t)0, (const Ctl*)nullptr);
+      full_launch<float, double>(P.p32, P.p32.vin, P.w, nullptr, 1.0, 0.0, nullptr, 0, nullptr, P.stream);
     } else {
-      launch(k_fullmv<double, double, double>, P.op64.gU + P.op64.gP + P.op64.gS, 128, 0, P.stream, P.op64, tmp, P.w,
-             nullptr, 1.0, 0.0, (double*)nullptr, (size_t)0, (const Ctl*)nullptr);
+      full_launch<double, double>(P.p64, tmp, P.w, nullptr, 1.0, 0.0, nullptr, 0, nullptr, P.stream);
     }
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(yh, P.w, P.n * 8, cudaMemcpyDeviceToHost, P.stream));
@@ -2902,14 +2992,12 @@ int fsi_time_kernel(fsi_problem* h, int which, int reps, double* avg_ms, double*
       CK(cudaEventRecord(e0, s));
       switch (which) {
         case 0:  // full operator, FP32 (mixed inner iteration)
-          launch(k_fullmv<float, float, double>, P.op32.gU + P.op32.gP + P.op32.gS, 128, 0, s, P.op32, P.p32.zw, P.w,
-                 nullptr, 1.0, 0.0, (float*)nullptr, (size_t)0, (const Ctl*)nullptr);
-          *bytes = fullop_bytes<float>(P, cfnnz, sizeof(float), sizeof(double));
+          full_launch<float, double>(P.p32, P.p32.zw, P.w, nullptr, 1.0, 0.0, nullptr, 0, nullptr, s);
+          *bytes = fullop_bytes<float>(P, P.p32.mf.N > 0, cfnnz, sizeof(float), sizeof(double));
           break;
         case 1:  // full operator, FP64 (residual / FP64 iteration)
-          launch(k_fullmv<double, double, double>, P.op64.gU + P.op64.gP + P.op64.gS, 128, 0, s, P.op64, P.x, P.w, P.b,
-                 -1.0, 1.0, (double*)nullptr, (size_t)0, (const Ctl*)nullptr);
-          *bytes = fullop_bytes<double>(P, cfnnz, 16, 8);
+          full_launch<double, double>(P.p64, P.x, P.w, P.b, -1.0, 1.0, nullptr, 0, nullptr, s);
+          *bytes = fullop_bytes<double>(P, P.p64.mf.N > 0, cfnnz, 16, 8);
           break;
         case 2: {  // finest velocity Chebyshev step, FP32
           MGLevel<float>& L = P.p32.mgU.lv[0];
