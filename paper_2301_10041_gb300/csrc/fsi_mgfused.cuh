@@ -89,8 +89,11 @@ constexpr int mf_pres_blk(int v, int y, int x) { return kMfPresVar * v + kMfPres
 // the overlaps the tiles repeat: on the 128 x 128 cavity, tiles shrunk to
 // keep 256 CTAs on every level measured slower (9.8 against 10.7 steps/s)
 // than one tile size for all levels.  From 512 cells on, the larger tiles
-// repeat less of their neighbours' work.
-__host__ __device__ __forceinline__ int mf_tile_u(int N) { return N >= 512 ? 16 : 8; }
+// repeat less of their neighbours' work.  Up to 32 cells a velocity level takes
+// 4-node tiles: 64 CTAs of 384 threads instead of 16 of 512, down 3.35 -> 3.0 us,
+// up 3.3 -> 2.9 us on 32 cells (but 3.4 -> 5.8 us on 64, where they do not all fit
+// beside their four times repeated overlap).
+__host__ __device__ __forceinline__ int mf_tile_u(int N) { return N >= 512 ? 16 : (N > 32 ? 8 : 4); }
 __host__ __device__ __forceinline__ int mf_tile_p(int N) { return N >= 512 ? 8 : 4; }
 // Threads of a velocity launch.  A launch's time on these grids is one CTA's
 // chain of phases, and the threads' share of a phase sets it.  The stencil
@@ -100,7 +103,7 @@ __host__ __device__ __forceinline__ int mf_tile_p(int N) { return N >= 512 ? 8 :
 // grids use 512 as well (1024 measured slower there).  Down frames have
 // TC + 8 plane entries a side (four planes), up frames TC + 4; a warp takes
 // two rows of up to 16 entries, four rows of up to 8.
-constexpr int mf_threads_ud(int tc) { return tc >= 16 ? 512 : (tc == 8 ? 512 : (tc == 4 ? 768 : 640)); }
+constexpr int mf_threads_ud(int tc) { return tc >= 16 ? 512 : (tc == 8 ? 512 : (tc == 4 ? 384 : 640)); }
 constexpr int mf_threads_uu(int tc) { return tc >= 16 ? 512 : (tc == 8 ? 512 : (tc == 4 ? 256 : 192)); }
 constexpr int mf_threads_p(int tp) { return tp >= 4 ? 256 : 128; }
 
@@ -149,6 +152,10 @@ template <class T>
 struct MfVelOp {
   int N = 0;
   T c[4][5][5][4];
+  // the same as (c0, c3, c1, c1) for the packed FP32 multiply-adds: the blocks
+  // are symmetric with equal off-diagonal entries, zero for two nodes on one grid
+  // line (the caller fills it and checks that; device code reads no other)
+  alignas(16) T pk[4][5][5][4] = {};
   T dinv[4][2];
 };
 
@@ -321,8 +328,45 @@ __host__ __device__ __forceinline__ int mf_vnode(int N, int ix, int iy) {
   }
 }
 
+// the same with the type as a value
+__host__ __device__ __forceinline__ int mf_vnode_rt(int N, int t, int ix, int iy) {
+  const int nV = (N - 1) * (N - 1), nX = N * (N - 1);
+  const int off = t == 0 ? 0 : (t == 1 ? nV : (t == 2 ? nV + nX : nV + 2 * nX));
+  return off + ((iy >> 1) - 1 + (t >> 1)) * (N - 1 + (t & 1)) + (ix >> 1) - 1 + (t & 1);
+}
+
 __host__ __device__ __forceinline__ bool mf_vinterior(int N, int ix, int iy) {
   return ix >= 1 && iy >= 1 && ix <= 2 * N - 1 && iy <= 2 * N - 1;
+}
+
+// Loading a frame.  fn(slot, entry, type, ix, iy) for the entries e = t, t + NT,
+// ... of a frame of four planes of PW x PW entries, slot = 0, 1, ...: a thread
+// first loads all its entries into registers, then stores them, so a frame costs
+// one memory round trip.  (A sweep that loads and stores entry by entry exposed
+// one per round: 5 rounds, 3 us, for the start of a residual launch.)
+template <int PW, int NT, class F>
+__host__ __device__ __forceinline__ void mf_entries(int t, int ox, int oy, F&& fn) {
+  constexpr int n = 4 * PW * PW, R = (n + NT - 1) / NT;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int e = t + r * NT;
+    if (e >= n) continue;
+    const int ty = e / (PW * PW), q = e - ty * (PW * PW), py = q / PW, px = q - py * PW;
+    fn(r, e, ty, ox + 2 * px + (ty & 1), oy + 2 * py + (ty >> 1));
+  }
+}
+constexpr int mf_rounds(int pw, int nt) { return (4 * pw * pw + nt - 1) / nt; }
+
+// the value of vector v (node order) at the lattice node (ix, iy) of type t,
+// zero on the wall and outside
+template <class T>
+__host__ __device__ __forceinline__ typename Vec2<T>::type mf_node_value(const T* __restrict__ v, int N, int t, int ix,
+                                                                         int iy) {
+  typename Vec2<T>::type x;
+  x.x = x.y = 0;
+  if (mf_vinterior(N, ix, iy))
+    x = *reinterpret_cast<const typename Vec2<T>::type*>(v + 2 * (size_t)mf_vnode_rt(N, t, ix, iy));
+  return x;
 }
 
 // a b + c in one rounding on the device (a multiply-add the stencil sums are
@@ -360,16 +404,62 @@ struct MfFrameT {
   }
 };
 
+#ifdef __CUDA_ARCH__
+// two FP32 multiply-adds in one instruction: lanes of d = a * b + c
+__device__ __forceinline__ unsigned long long mf_fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ float2 mf_unpack(unsigned long long a) {
+  return make_float2(__uint_as_float((unsigned)a), __uint_as_float((unsigned)(a >> 32)));
+}
+#endif
+
 // y = A v at the node of type TAU with plane coordinates (px, py) of frame
 // f; the neighbours of even and odd rows go to two accumulator pairs (two
-// shorter dependency chains of multiply-adds), added at the end
+// shorter dependency chains of multiply-adds), added at the end.  In FP32 on
+// the device the products are packed, with the node's (x, y) pair as it lies in
+// shared memory: (c0 x, c3 y), and off the axes (c1 x, c1 y), whose halves swap
+// at the very end.  25 packed multiply-adds a node on average instead of 64
+// plain ones, and one constant load per block.
 template <class T, int TAU, class F>
 __host__ __device__ __forceinline__ void mf_vel_apply(const MfVelOp<T>& op, const typename Vec2<T>::type* __restrict__ v,
                                                       const F& f, int px, int py, T& y0, T& y1) {
   constexpr int PX = TAU & 1, PY = TAU >> 1;
   constexpr int RX = PX ? 1 : 2, RY = PY ? 1 : 2;
-  T a0 = 0, a1 = 0, b0 = 0, b1 = 0;
   const typename Vec2<T>::type* __restrict__ w = v + f.at(0, px, py);
+#ifdef __CUDA_ARCH__
+  if constexpr (std::is_same<T, float>::value) {
+    // per tap (x, y) += (c0 x, c3 y); off the axes also (c1 x, c1 y), whose
+    // halves swap at the end
+    unsigned long long p0 = 0, p1 = 0, q0 = 0, q1 = 0;
+#pragma unroll
+    for (int dy = -RY; dy <= RY; ++dy) {
+#pragma unroll
+      for (int dx = -RX; dx <= RX; ++dx) {
+        const int t2 = ((PX + dx) & 1) | (((PY + dy) & 1) << 1);
+        const unsigned long long x = *reinterpret_cast<const unsigned long long*>(
+            w + (t2 * f.ph + ((PY + dy) >> 1)) * f.pw + ((PX + dx) >> 1));
+        const float* c = op.pk[TAU][dy + 2][dx + 2];
+        if (dx == 0 || dy == 0) {
+          const unsigned long long cd = *reinterpret_cast<const unsigned long long*>(c);
+          if ((dy & 1) == 0) p0 = mf_fma2(cd, x, p0);
+          else q0 = mf_fma2(cd, x, q0);
+        } else {
+          const ulonglong2 cc = *reinterpret_cast<const ulonglong2*>(c);
+          if ((dy & 1) == 0) { p0 = mf_fma2(cc.x, x, p0); p1 = mf_fma2(cc.y, x, p1); }
+          else { q0 = mf_fma2(cc.x, x, q0); q1 = mf_fma2(cc.y, x, q1); }
+        }
+      }
+    }
+    const float2 d0 = mf_unpack(p0), d1 = mf_unpack(q0), e0 = mf_unpack(p1), e1 = mf_unpack(q1);
+    y0 = (d0.x + d1.x) + (e0.y + e1.y);
+    y1 = (d0.y + d1.y) + (e0.x + e1.x);
+    return;
+  }
+#endif
+  T a0 = 0, a1 = 0, b0 = 0, b1 = 0;
 #pragma unroll
   for (int dy = -RY; dy <= RY; ++dy) {
 #pragma unroll
@@ -487,70 +577,106 @@ __host__ __device__ void mfu_down_body(const MfVelArgs<T>& a, const MfCta& cta) 
   g.oy = f.oy - 2;
   T2* Z = Dn;
   static_assert(TC + 4 + 2 * K >= 8, "the grown frame must fit in Dn and R");
-  // With zu, the frame's b and the pressure of the cells around the frame
-  // (cells f.ox / 2 - 1 .. f.ox / 2 + PW - 1, PW + 1 a side, after Z when they
-  // fit) come in the same phase, so the launch makes one global round trip
-  // before its first barrier.
+  // The frame's b, and with zu the iterate and the pressure of the cells around
+  // the frame (cells f.ox / 2 - 1 .. f.ox / 2 + PW - 1, PW + 1 a side, after Z
+  // when they fit), come in one phase of loads that are all in flight at once.
   constexpr int ZPW = PW + 1;
   constexpr bool zp_frame = 4 * (PW + 2) * (PW + 2) * 2 + 3 * ZPW * ZPW <= 2 * nf * 2;
   T* ZP = reinterpret_cast<T*>(Z + 4 * (PW + 2) * (PW + 2));
   const int zcx0 = (f.ox >> 1) - 1, zcy0 = (f.oy >> 1) - 1;
   const bool zp_smem = zp_frame && rs.zu && rs.zp;
-  if (rs.zu) {
-    mf_vsweep(cta, 0, g.pw, 0, g.ph, [&](auto tc, int px, int py) {
-      constexpr int TAU = decltype(tc)::value;
-      const int ix = g.ox + 2 * px + (TAU & 1), iy = g.oy + 2 * py + (TAU >> 1);
-      T2 v;
-      v.x = v.y = 0;
-      if (mf_vinterior(N, ix, iy)) v = *reinterpret_cast<const T2*>(rs.zu + 2 * (size_t)mf_vnode_t<TAU>(N, ix, iy));
-      Z[g.at(TAU, px, py)] = v;
+  constexpr int NT = mf_threads_ud(TC);
+  for (int t = cta.tid; t < NT; t += cta.nthr) {
+    T2 zv[mf_rounds(PW + 2, NT)], bv[mf_rounds(PW, NT)];
+    constexpr int RZ = (ZPW * ZPW + NT - 1) / NT;
+    T pv[RZ][3];
+    if (rs.zu) mf_entries<PW + 2, NT>(t, g.ox, g.oy, [&](int r, int, int ty, int ix, int iy) {
+      zv[r] = mf_node_value<T>(rs.zu, N, ty, ix, iy);
     });
-    mf_vsweep(cta, 0, f.pw, 0, f.ph, [&](auto tc, int px, int py) {
-      constexpr int TAU = decltype(tc)::value;
-      const int ix = f.ox + 2 * px + (TAU & 1), iy = f.oy + 2 * py + (TAU >> 1);
-      T2 v;
-      v.x = v.y = 0;
-      if (mf_vinterior(N, ix, iy)) v = *reinterpret_cast<const T2*>(a.b + 2 * (size_t)mf_vnode_t<TAU>(N, ix, iy));
-      B[f.at(TAU, px, py)] = v;
+    mf_entries<PW, NT>(t, f.ox, f.oy, [&](int r, int, int ty, int ix, int iy) {
+      bv[r] = mf_node_value<T>(a.b, N, ty, ix, iy);
     });
-    if (zp_smem)
-      mf_rows(cta, ZPW, ZPW, [&](int i, int j) {
-        const int cx = zcx0 + i, cy = zcy0 + j;
-        const bool in = cx >= 0 && cy >= 0 && cx < N && cy < N;
+    if (zp_smem) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) ZP[3 * (j * ZPW + i) + k] = in ? rs.zp[3 * ((size_t)cy * N + cx) + k] : (T)0;
-      });
-    MF_SYNC();
-  }
-  // b on the frame (with the residual start: b - A zu - (-B^T) zp, its owned
-  // part to rs.bout); x0 = d0 = c0 D^-1 b
-  mf_vsweep(cta, 0, f.pw, 0, f.ph, [&](auto tc, int px, int py) {
-    constexpr int TAU = decltype(tc)::value;
-    const int ix = f.ox + 2 * px + (TAU & 1), iy = f.oy + 2 * py + (TAU >> 1);
-    const int e = f.at(TAU, px, py);
-    T2 v;
-    v.x = v.y = 0;
-    if (mf_vinterior(N, ix, iy)) {
-      const size_t id = 2 * (size_t)mf_vnode_t<TAU>(N, ix, iy);
-      v = rs.zu ? B[e] : *reinterpret_cast<const T2*>(a.b + id);
-      if (rs.zu || rs.zp) {
-        T y0 = 0, y1 = 0;
-        if (rs.zu) mf_vel_apply<T, TAU>(op, Z, g, px + 1, py + 1, y0, y1);
-        if (zp_smem) mf_vel_btp<T, TAU>(rs, ZP, zcx0, zcy0, ZPW, ix, iy, y0, y1);
-        else if (rs.zp) mf_vel_btp<T, TAU>(rs, rs.zp, 0, 0, N, ix, iy, y0, y1);
-        v.x -= y0;
-        v.y -= y1;
-        if (px >= o && px < o + TC && py >= o && py < o + TC) *reinterpret_cast<T2*>(rs.bout + id) = v;
+      for (int r = 0; r < RZ; ++r) {
+        const int e = t + r * NT, j = e / ZPW, cx = zcx0 + e - j * ZPW, cy = zcy0 + j;
+        const bool in = e < ZPW * ZPW && cx >= 0 && cy >= 0 && cx < N && cy < N;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) pv[r][k] = in ? rs.zp[3 * ((size_t)cy * N + cx) + k] : (T)0;
       }
     }
+    if (rs.zu) mf_entries<PW + 2, NT>(t, g.ox, g.oy, [&](int r, int e, int, int, int) { Z[e] = zv[r]; });
+    mf_entries<PW, NT>(t, f.ox, f.oy, [&](int r, int e, int ty, int, int) {
+      B[e] = bv[r];
+      if (!rs.zu && !rs.zp) {   // the right-hand side as it is: the smoother starts here
+        T2 x0;
+        x0.x = a.ch.c0 * op.dinv[ty][0] * bv[r].x;
+        x0.y = a.ch.c0 * op.dinv[ty][1] * bv[r].y;
+        Xc[e] = x0;
+        Dc[e] = x0;
+      }
+    });
+    if (zp_smem) {
+#pragma unroll
+      for (int r = 0; r < RZ; ++r) {
+        const int e = t + r * NT;
+        if (e < ZPW * ZPW) {
+#pragma unroll
+          for (int k = 0; k < 3; ++k) ZP[3 * e + k] = pv[r][k];
+        }
+      }
+    }
+  }
+  MF_SYNC();
+  // b on the frame (with the residual start: b - A zu - (-B^T) zp, its owned
+  // part to rs.bout); x0 = d0 = c0 D^-1 b
+  auto start = [&](auto tc, int px, int py, int ix, int iy, T2 v) {
+    constexpr int TAU = decltype(tc)::value;
+    const int e = f.at(TAU, px, py);
     B[e] = v;
     T2 x0;
     x0.x = a.ch.c0 * op.dinv[TAU][0] * v.x;
     x0.y = a.ch.c0 * op.dinv[TAU][1] * v.y;
     Xc[e] = x0;
     Dc[e] = x0;
-  });
-  MF_SYNC();
+    if (mf_vinterior(N, ix, iy) && px >= o && px < o + TC && py >= o && py < o + TC)
+      *reinterpret_cast<T2*>(rs.bout + 2 * (size_t)mf_vnode_t<TAU>(N, ix, iy)) = v;
+  };
+  if (rs.zu)
+    mf_vsweep2(cta, 0, f.pw, 0, f.ph, [&](auto tc, int px, int py) {   // two plane rows per thread, as the smoothing
+      constexpr int TAU = decltype(tc)::value;
+      T y[2][2];
+      mf_vel_apply<T, TAU>(op, Z, g, px + 1, py + 1, y[0][0], y[0][1]);
+      mf_vel_apply<T, TAU>(op, Z, g, px + 1, py + 2, y[1][0], y[1][1]);
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int qy = py + k, ix = f.ox + 2 * px + (TAU & 1), iy = f.oy + 2 * qy + (TAU >> 1);
+        T2 v;
+        v.x = v.y = 0;
+        if (mf_vinterior(N, ix, iy)) {
+          v = B[f.at(TAU, px, qy)];
+          if (zp_smem) mf_vel_btp<T, TAU>(rs, ZP, zcx0, zcy0, ZPW, ix, iy, y[k][0], y[k][1]);
+          else if (rs.zp) mf_vel_btp<T, TAU>(rs, rs.zp, 0, 0, N, ix, iy, y[k][0], y[k][1]);
+          v.x -= y[k][0];
+          v.y -= y[k][1];
+        }
+        start(tc, px, qy, ix, iy, v);
+      }
+    });
+  else if (rs.zp)
+    mf_vsweep(cta, 0, f.pw, 0, f.ph, [&](auto tc, int px, int py) {
+      constexpr int TAU = decltype(tc)::value;
+      const int ix = f.ox + 2 * px + (TAU & 1), iy = f.oy + 2 * py + (TAU >> 1);
+      T2 v = B[f.at(TAU, px, py)];
+      if (mf_vinterior(N, ix, iy)) {
+        T y0 = 0, y1 = 0;
+        mf_vel_btp<T, TAU>(rs, rs.zp, 0, 0, N, ix, iy, y0, y1);
+        v.x -= y0;
+        v.y -= y1;
+      }
+      start(tc, px, py, ix, iy, v);
+    });
+  if (rs.zu || rs.zp) MF_SYNC();
   for (int s = 1; s < K; ++s) {  // pre-smoothing steps 1 .. K-1 on the frame shrunk by s nodes per plane
     mf_vel_cheb<T>(cta, op, f, s, B, Xc, Dc, Xn, Dn, false, a.ch.c1[s - 1], a.ch.c2[s - 1]);
     T2* t = Xc; Xc = Xn; Xn = t;
@@ -649,61 +775,59 @@ __host__ __device__ void mfu_up_body(const MfVelArgs<T>& a, const MfCta& cta) {
   f.ox = FX0 - 2 * K;
   f.oy = FY0 - 2 * K;
   // coarse lattice frame covering the prolongation taps of the fine frame
-  MfFrame g;
-  {
-    const int lox = mf_max(f.ox, 0) >> 2, loy = mf_max(f.oy, 0) >> 2;
-    const int hix = mf_min((f.ox + 2 * f.pw - 1) >> 2, Nc - 1), hiy = mf_min((f.oy + 2 * f.ph - 1) >> 2, Nc - 1);
-    g.ox = 2 * lox;
-    g.oy = 2 * loy;
-    g.pw = hix - lox + 2;   // coarse lattice 2 lo .. 2 hi + 2, i.e. 2 (hi - lo) + 3 nodes
-    g.ph = hiy - loy + 2;
-  }
+  // (the coarse cells f.ox / 4 .. (f.ox + 2 PW - 1) / 4 and one node more)
+  constexpr int GP = (2 * PW + 3) / 4 + 2;
+  MfFrameT<GP, GP> g;
+  g.ox = 2 * (f.ox >> 2);
+  g.oy = 2 * (f.oy >> 2);
   constexpr int nf = 4 * PW * PW;
   T2* B = reinterpret_cast<T2*>(cta.sm);
   T2 *Xc = B + nf, *Xn = B + 2 * nf, *Dc = B + 3 * nf, *Dn = B + 4 * nf;
   T2* XC = B + 5 * nf;
-  mf_vsweep(cta, 0, g.pw, 0, g.ph, [&](auto tc, int px, int py) {
-    constexpr int TAU = decltype(tc)::value;
-    const int ix = g.ox + 2 * px + (TAU & 1), iy = g.oy + 2 * py + (TAU >> 1);
-    T2 v;
-    v.x = v.y = 0;
-    if (mf_vinterior(Nc, ix, iy)) v = *reinterpret_cast<const T2*>(a.xc + 2 * (size_t)mf_vnode_t<TAU>(Nc, ix, iy));
-    XC[g.at(TAU, px, py)] = v;
-  });
+  // b, the pre-smoothed iterate and the coarse correction, all in flight at once
+  constexpr int NT = mf_threads_uu(TC);
+  for (int t = cta.tid; t < NT; t += cta.nthr) {
+    T2 cv[mf_rounds(GP, NT)], bv[mf_rounds(PW, NT)], xv[mf_rounds(PW, NT)];
+    mf_entries<GP, NT>(t, g.ox, g.oy, [&](int r, int, int ty, int ix, int iy) {
+      cv[r] = mf_node_value<T>(a.xc, Nc, ty, ix, iy);
+    });
+    mf_entries<PW, NT>(t, f.ox, f.oy, [&](int r, int, int ty, int ix, int iy) {
+      bv[r] = mf_node_value<T>(a.b, N, ty, ix, iy);
+      xv[r] = mf_node_value<T>(a.xpre, N, ty, ix, iy);
+    });
+    mf_entries<GP, NT>(t, g.ox, g.oy, [&](int r, int e, int, int, int) { XC[e] = cv[r]; });
+    mf_entries<PW, NT>(t, f.ox, f.oy, [&](int r, int e, int, int, int) {
+      B[e] = bv[r];
+      Xc[e] = xv[r];
+    });
+  }
   MF_SYNC();
-  // b and x + P x_coarse on the frame: the coarse quadratic of the coarse
-  // cell cc = min(ix / 4, Nc - 1) at t = (ix - 4 cc) / 4 in each direction
-  mf_vsweep(cta, 0, f.pw, 0, f.ph, [&](auto tc, int px, int py) {
-    constexpr int TAU = decltype(tc)::value;
-    const int ix = f.ox + 2 * px + (TAU & 1), iy = f.oy + 2 * py + (TAU >> 1);
-    T2 bv, xv;
-    bv.x = bv.y = xv.x = xv.y = 0;
-    if (mf_vinterior(N, ix, iy)) {
-      const size_t id = mf_vnode_t<TAU>(N, ix, iy);
-      bv = *reinterpret_cast<const T2*>(a.b + 2 * id);
-      xv = *reinterpret_cast<const T2*>(a.xpre + 2 * id);
-      const int ccx = mf_min(ix >> 2, Nc - 1), ccy = mf_min(iy >> 2, Nc - 1);
-      const float tx = 0.25f * (float)(ix - 4 * ccx), ty = 0.25f * (float)(iy - 4 * ccy);
+  // x + P x_coarse on the frame: the coarse quadratic of the coarse cell
+  // cc = ix / 4 at t = (ix - 4 cc) / 4 in each direction (interior nodes have
+  // ix <= 2 N - 1, so cc < Nc)
+  for (int t = cta.tid; t < NT; t += cta.nthr)
+    mf_entries<PW, NT>(t, f.ox, f.oy, [&](int, int e, int, int ix, int iy) {
+      if (!mf_vinterior(N, ix, iy)) return;
+      const float tx = 0.25f * (float)(ix & 3), ty = 0.25f * (float)(iy & 3);
       const T wx[3] = {(T)mf_l0(tx), (T)mf_l1(tx), (T)mf_l2(tx)};
       const T wy[3] = {(T)mf_l0(ty), (T)mf_l1(ty), (T)mf_l2(ty)};
+      const int px = ((ix >> 2) * 2 - g.ox) >> 1, py = ((iy >> 2) * 2 - g.oy) >> 1;
       T p0 = 0, p1 = 0;
 #pragma unroll
       for (int bb = 0; bb < 3; ++bb) {
 #pragma unroll
         for (int aa = 0; aa < 3; ++aa) {
           const T w = wx[aa] * wy[bb];
-          const T2 c = XC[g.at_lattice(2 * ccx + aa, 2 * ccy + bb)];
+          const T2 c = XC[g.at((aa & 1) | ((bb & 1) << 1), px + (aa >> 1), py + (bb >> 1))];
           p0 += w * c.x;
           p1 += w * c.y;
         }
       }
-      xv.x = p0 + xv.x;
-      xv.y = p1 + xv.y;
-    }
-    const int e = f.at(TAU, px, py);
-    B[e] = bv;
-    Xc[e] = xv;
-  });
+      T2 x = Xc[e];
+      x.x += p0;
+      x.y += p1;
+      Xc[e] = x;
+    });
   MF_SYNC();
   // The Richardson update of the last step reads the iterate it adds to.
   // With K >= 2 those reads go out in the phase before the last step, into
@@ -1058,20 +1182,26 @@ __host__ __device__ void mfp_up_body(const MfPresArgs<T>& a, const MfCta& cta) {
 
 #ifdef __CUDACC__
 // The kernels: one CTA per tile, NT threads.
-#define FSI_MF_KERNEL(name, body, Args)                                                      \
+// MINB: CTAs per SM the registers must leave room for.  Velocity: two, since the
+// 128-cell level has 256 CTAs for 152 SMs (one per SM cost 4.9 -> 6.7 us there).
+#define FSI_MF_BOUNDS_V __launch_bounds__(NT, TILE >= 8 ? 2 : 1)
+#define FSI_MF_BOUNDS_P __launch_bounds__(NT)
+#define FSI_MF_KERNEL(name, body, Args, BOUNDS)                                              \
   template <class T, int TILE, int K, int NT>                                                \
-  __global__ void __launch_bounds__(NT) name(const __grid_constant__ Args<T> a) {            \
+  __global__ void BOUNDS name(const __grid_constant__ Args<T> a) {            \
     asm volatile("griddepcontrol.wait;" ::: "memory");                                       \
     extern __shared__ __align__(16) unsigned char mf_smem[];                                 \
     const MfCta c{(int)blockIdx.x, (int)blockIdx.y, (int)threadIdx.x, (int)blockDim.x, NT,   \
                   mf_smem};                                                                  \
     body<T, TILE, K>(a, c);                                                                  \
   }
-FSI_MF_KERNEL(k_mfu_down, mfu_down_body, MfVelArgs)
-FSI_MF_KERNEL(k_mfu_up, mfu_up_body, MfVelArgs)
-FSI_MF_KERNEL(k_mfp_down, mfp_down_body, MfPresArgs)
-FSI_MF_KERNEL(k_mfp_up, mfp_up_body, MfPresArgs)
+FSI_MF_KERNEL(k_mfu_down, mfu_down_body, MfVelArgs, FSI_MF_BOUNDS_V)
+FSI_MF_KERNEL(k_mfu_up, mfu_up_body, MfVelArgs, FSI_MF_BOUNDS_V)
+FSI_MF_KERNEL(k_mfp_down, mfp_down_body, MfPresArgs, FSI_MF_BOUNDS_P)
+FSI_MF_KERNEL(k_mfp_up, mfp_up_body, MfPresArgs, FSI_MF_BOUNDS_P)
 #undef FSI_MF_KERNEL
+#undef FSI_MF_BOUNDS_V
+#undef FSI_MF_BOUNDS_P
 #endif
 
 // shared memory of one launch (bytes) for tile tc (velocity: coarse lattice

@@ -314,6 +314,7 @@ struct MGLevel {
   // and whether the V-cycle runs them on this level
   bool mf = false;
   MfVelOp<T> mfu;        // velocity hierarchy
+  bool mf_ok = false;    // the stencils have the form the kernels use
   T* mftab = nullptr;    // pressure hierarchy: kMfPresTab values
   MfOp<T> mfo;           // velocity hierarchy: the level's product matrix-free (mfo.N > 0)
   bool mfl = false;      // pressure hierarchy: the same, from mftab
@@ -490,10 +491,15 @@ static void build_mg(Arena& ar, const HostSetup& hs, bool pressure, int degree, 
           for (int d = 0; d < 2; ++d) L.divB[k][q][d] = (T)H.divB[k][q][d];
     if (H.mf && !pressure) {
       L.mfu.N = H.N;
+      L.mf_ok = make_mfop<T>(H).N > 0;
       for (int t = 0; t < 4; ++t) {
         for (int y = 0; y < 5; ++y)
           for (int x = 0; x < 5; ++x)
-            for (int q = 0; q < 4; ++q) L.mfu.c[t][y][x][q] = (T)H.stenA[t][y][x][q];
+            for (int q = 0; q < 4; ++q) {
+              L.mfu.c[t][y][x][q] = (T)H.stenA[t][y][x][q];
+              constexpr int kPack[4] = {0, 3, 1, 1};
+              L.mfu.pk[t][y][x][q] = (T)H.stenA[t][y][x][kPack[q]];
+            }
         for (int c = 0; c < 2; ++c) L.mfu.dinv[t][c] = (T)H.dinvAt[t][c];
       }
     } else if (H.mf) {
@@ -505,6 +511,7 @@ static void build_mg(Arena& ar, const HostSetup& hs, bool pressure, int degree, 
       for (int v = 0; v < 9; ++v)
         for (int k = 0; k < 3; ++k) tab[kMfPresDinv + 3 * v + k] = H.dinvLv[v][k];
       L.mftab = upload_as<T>(ar, tab);
+      L.mf_ok = true;
       L.mfl = mfree && H.N >= kMfo64MinN;
     }
     if (mfree && !pressure && H.N >= kMfo64MinN) L.mfo = make_mfop<T>(H);
@@ -599,7 +606,7 @@ static void select_mf(MG<T>& mg, const HostSetup& hs, int mg_fused, bool count_o
   bool any = false;
   for (int l = 0; l < last; ++l) {
     if (mg.cl.on && l >= mg.cl.lc) break;
-    if (!hs.levels[l].mf || hs.levels[l].N < 16) break;
+    if (!mg.lv[l].mf_ok || hs.levels[l].N < 16) break;
     mg.lv[l].mf = true;
     any = true;
   }
