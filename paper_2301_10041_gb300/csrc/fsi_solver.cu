@@ -956,6 +956,7 @@ struct Problem {
   Ctl* ctl = nullptr;
   Ctl* ctl_host = nullptr;   // pinned mirror
   int red_blocks = 0;
+  bool gs_cluster = false;   // the orthogonalisation runs as one cluster (small problems)
   // preconditioners
   Prec<double> p64;
   Prec<float> p32;
@@ -1527,17 +1528,30 @@ struct KrylovArgs {
 struct ArnoldiShared {
   double h[256], cb[256], ns[256], a[256];   // column, c b, -s, partly rotated a
 };
-
-__device__ __forceinline__ void arnoldi_finish(const KrylovArgs& k, ArnoldiShared& sh, const double* h2s, double s2) {
-  Ctl* c = k.ctl;
-  const int j = c->j, m1 = c->m + 1, t = threadIdx.x;   // j < 250 <= the CTA's threads
-  double cst = 0, snt = 0;
-  if (t <= j) sh.h[t] = k.h1[t] + (h2s ? h2s[t] : 0.0);
+// this thread's inputs of the Givens step, read by every CTA while it waits
+// for its rows anyway: only one CTA needs them, at the very end
+struct ArnoldiIn {
+  double h1 = 0, cs = 0, sn = 0, g = 0;
+};
+__device__ __forceinline__ ArnoldiIn arnoldi_load(const KrylovArgs& k, int j) {
+  const int t = threadIdx.x;   // j < 250 <= the CTA's threads
+  ArnoldiIn in;
+  if (t <= j) in.h1 = k.h1[t];
   if (t < j) {
-    cst = k.cs[t];
-    snt = k.sn[t];
-    sh.ns[t] = -snt;
+    in.cs = k.cs[t];
+    in.sn = k.sn[t];
   }
+  if (t == 0) in.g = k.g[j];
+  return in;
+}
+
+__device__ __forceinline__ void arnoldi_finish(const KrylovArgs& k, ArnoldiShared& sh, const ArnoldiIn& in, int j,
+                                               const double* h2s, double s2) {
+  Ctl* c = k.ctl;
+  const int m1 = c->m + 1, t = threadIdx.x;
+  const double cst = in.cs, snt = in.sn;
+  if (t <= j) sh.h[t] = in.h1 + (h2s ? h2s[t] : 0.0);
+  if (t < j) sh.ns[t] = -snt;
   __syncthreads();
   if (t < j) sh.cb[t] = cst * sh.h[t + 1];
   __syncthreads();
@@ -1555,7 +1569,7 @@ __device__ __forceinline__ void arnoldi_finish(const KrylovArgs& k, ArnoldiShare
     const double q0 = __shfl_sync(0xffffffffu, quo, 0), q1 = __shfl_sync(0xffffffffu, quo, 1);
     const double q2 = __shfl_sync(0xffffffffu, quo, 2);
     if (t == 0) {
-      const double gj = k.g[j];
+      const double gj = in.g;
       const double cc = (r > 0) ? q0 : 1.0, ss = (r > 0) ? q1 : 0.0;
       k.cs[j] = cc;
       k.sn[j] = ss;
@@ -1632,10 +1646,12 @@ __global__ void __launch_bounds__(kRedThreads, 3) k_gs2(KrylovArgs k) {
   __shared__ double hs[256], acc[256], sm[32];
   __shared__ ArnoldiShared ash;
   __shared__ double s2s;
-  const int cnt = k.ctl->j + 1, nb = gridDim.x;
-  for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
-    hs[i] = k.h1[i];
-    acc[i] = 0;
+  const int j = k.ctl->j, cnt = j + 1, nb = gridDim.x;
+  const ArnoldiIn in = arnoldi_load(k, j);
+  const double wn2 = threadIdx.x == 0 ? k.h1[cnt] : 0.0;
+  if (threadIdx.x < cnt) {
+    hs[threadIdx.x] = in.h1;
+    acc[threadIdx.x] = 0;
   }
   const int nsub = (k.n + CH - 1) / CH;
   double nacc = 0;
@@ -1663,13 +1679,13 @@ __global__ void __launch_bounds__(kRedThreads, 3) k_gs2(KrylovArgs k) {
       Ctl* c = k.ctl;
       c->counter[1] = 0;
       const double s2 = k.h2[cnt];
-      c->refine = (s2 < 0.5 * k.h1[cnt]) ? 1 : 0;
+      c->refine = (s2 < 0.5 * wn2) ? 1 : 0;
       if (c->refine) c->refines += 1;
       s2s = c->refine ? -1.0 : s2;
     }
     __syncthreads();
     // -1 marks the refinement; a NaN norm is not below any bound and finishes here
-    if (s2s != -1.0) arnoldi_finish(k, ash, nullptr, s2s);
+    if (s2s != -1.0) arnoldi_finish(k, ash, in, j, nullptr, s2s);
   }
 }
 
@@ -1680,9 +1696,10 @@ __global__ void __launch_bounds__(kRedThreads, 3) k_gs3(KrylovArgs k) {
   __shared__ double hs[256], sm[32];
   __shared__ ArnoldiShared ash;
   __shared__ double s2s;
-  if (!k.ctl->refine) return;
-  const int cnt = k.ctl->j + 1, nb = gridDim.x;
-  for (int i = threadIdx.x; i < cnt; i += blockDim.x) hs[i] = k.h2[i];
+  const int refine = k.ctl->refine, j = k.ctl->j, cnt = j + 1, nb = gridDim.x;
+  if (!refine) return;
+  const ArnoldiIn in = arnoldi_load(k, j);
+  if (threadIdx.x < cnt) hs[threadIdx.x] = k.h2[threadIdx.x];
   __syncthreads();
   const int nsub = (k.n + CH - 1) / CH;
   double nacc = 0;
@@ -1707,7 +1724,7 @@ __global__ void __launch_bounds__(kRedThreads, 3) k_gs3(KrylovArgs k) {
       s2s = s2;
     }
     __syncthreads();
-    arnoldi_finish(k, ash, hs, s2s);
+    arnoldi_finish(k, ash, in, j, hs, s2s);
   }
 }
 
@@ -1728,6 +1745,194 @@ __global__ void k_basis(int n2, double* __restrict__ V, size_t ld, const double*
   o.x = (T)v.x;
   o.y = (T)v.y;
   reinterpret_cast<typename Vec2<T>::type*>(vin)[i] = o;
+}
+
+// The whole orthogonalisation of a small problem in one launch: a cluster of 16
+// CTAs holds w in registers, sums its dots through distributed shared memory,
+// and goes through the same passes (h1 and ||w||, the update with h2, the
+// refinement if needed, the Givens step, the next basis vector) with cluster
+// barriers between them.  As launches, the passes of a 7400-unknown problem take
+// 33 us, nearly all of it launch boundaries, last-block hand-overs and the
+// FP64 latency of their reductions; 16 SMs hold the FP64 work of up to 1024
+// rows each (kGsClusterRows) in about the time the hand-overs take.
+// Rows are worked by four warps, one per SM quarter: an FP64 instruction holds
+// a quarter's pipe for 64 cycles, so more warps would only repeat the butterflies.
+constexpr int kGsCluster = 16;
+constexpr int kGsWorkers = 128;                       // threads that own row pairs
+constexpr int kGsPairs = 4;                           // row pairs of one of them, at most
+constexpr int kGsClusterRows = 2 * kGsWorkers * kGsPairs;
+
+struct GsClusterShared {
+  double red[4][260];          // per-warp sums
+  double part[3][260];         // this CTA's sums, read by the whole cluster
+  double h1[256], h2[260];     // the cluster's sums
+  double scale;
+};
+
+// sums of v over the cluster's CTAs: out[i] = sum_r part_r[i], i < cnt
+__device__ __forceinline__ void gs_cluster_gather(cg::cluster_group& cl, double* part, int cnt, double* out) {
+  const int r = threadIdx.x & 15;
+  const double* remote = cl.map_shared_rank(part, r);
+  for (int i0 = threadIdx.x >> 4; i0 - (int)(threadIdx.x >> 4) < cnt; i0 += 2 * (kRedThreads / 16)) {
+    const int i1 = i0 + kRedThreads / 16;
+    double a = i0 < cnt ? remote[i0] : 0.0, b = i1 < cnt ? remote[i1] : 0.0;
+    // two sums share the butterfly over 16 lanes: a in lanes 0-7, b in 8-15
+    const bool hi = r & 8;
+    double s = (hi ? b : a) + __shfl_xor_sync(0xffffffffu, hi ? a : b, 8);
+    s += __shfl_xor_sync(0xffffffffu, s, 4);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    if (r == 0 && i0 < cnt) out[i0] = s;
+    if (r == 8 && i1 < cnt) out[i1] = s;
+  }
+}
+
+// dots of this CTA's rows with V[0 .. cnt-1] and their sum of squares (entry
+// cnt), into part; every thread of the CTA calls it
+__device__ __forceinline__ void gs_cluster_dots(const double2* __restrict__ v0, size_t l2, int cnt, int np,
+                                                const double2* w, GsClusterShared& sh, double* part, bool dots) {
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  if (threadIdx.x < kGsWorkers) {
+    double nn = 0;
+#pragma unroll
+    for (int u = 0; u < kGsPairs; ++u) {
+      nn = fma(w[u].x, w[u].x, nn);
+      nn = fma(w[u].y, w[u].y, nn);
+    }
+    for (int i = 0; i < (dots ? cnt : 0) + 1; i += 4) {   // one slot past the vectors: the sum of squares
+      double a[4] = {0, 0, 0, 0};
+      const int nv = dots ? cnt : 0;
+#pragma unroll
+      for (int u = 0; u < kGsPairs; ++u) {
+        const int r = threadIdx.x + kGsWorkers * u;
+        if (r >= np) break;
+        double2 x[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (i + q < nv) x[q] = v0[(size_t)(i + q) * l2 + r];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (i + q < nv) a[q] = fma(x[q].y, w[u].y, fma(x[q].x, w[u].x, a[q]));
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (i + q == nv) a[q] = nn;
+      const double s = warp_sum4(a[0], a[1], a[2], a[3]);
+      const int mine = i + (lane >> 3);
+      if ((lane & 7) == 0 && mine <= nv) sh.red[wp][mine] = s;
+    }
+  }
+  __syncthreads();
+  const int nv = dots ? cnt : 0;
+  for (int i = threadIdx.x; i <= nv; i += kRedThreads)
+    part[i] = (sh.red[0][i] + sh.red[1][i]) + (sh.red[2][i] + sh.red[3][i]);
+}
+
+template <class T>
+__global__ void __launch_bounds__(kRedThreads) k_gs_cluster(KrylovArgs k, double* __restrict__ V, T* __restrict__ vin) {
+  pdl_begin();
+  __shared__ GsClusterShared sh;
+  __shared__ ArnoldiShared ash;
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank(), t = threadIdx.x;
+  const int j = k.ctl->j, cnt = j + 1;
+  const ArnoldiIn in = [&] {
+    ArnoldiIn v;
+    if (rank == 0) {
+      if (t < j) {
+        v.cs = k.cs[t];
+        v.sn = k.sn[t];
+      }
+      if (t == 0) v.g = k.g[j];
+    }
+    return v;
+  }();
+  const int n2 = k.n / 2, per = (n2 + kGsCluster - 1) / kGsCluster;   // row pairs of a CTA
+  const int p0 = min(n2, rank * per), np = min(n2, p0 + per) - p0;
+  const size_t l2 = k.ld >> 1;
+  const double2* __restrict__ v0 = reinterpret_cast<const double2*>(k.V) + p0;
+  double2 w[kGsPairs];
+#pragma unroll
+  for (int u = 0; u < kGsPairs; ++u) {
+    const int r = t + kGsWorkers * u;
+    w[u].x = w[u].y = 0;
+    if (t < kGsWorkers && r < np) w[u] = reinterpret_cast<const double2*>(k.w)[p0 + r];
+  }
+  auto update = [&](const double* h) {
+    if (t >= kGsWorkers) return;
+    for (int i = 0; i < cnt; i += 4) {
+#pragma unroll
+      for (int u = 0; u < kGsPairs; ++u) {
+        const int r = t + kGsWorkers * u;
+        if (r >= np) break;
+        double2 x[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (i + q < cnt) x[q] = v0[(size_t)(i + q) * l2 + r];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (i + q < cnt) {
+            w[u].x = fma(-h[i + q], x[q].x, w[u].x);
+            w[u].y = fma(-h[i + q], x[q].y, w[u].y);
+          }
+      }
+    }
+  };
+  gs_cluster_dots(v0, l2, cnt, np, w, sh, sh.part[0], true);
+  cl.sync();
+  gs_cluster_gather(cl, sh.part[0], cnt + 1, sh.h2);
+  __syncthreads();
+  const double wn2 = sh.h2[cnt];
+  if (t < cnt) sh.h1[t] = sh.h2[t];
+  __syncthreads();
+  update(sh.h1);
+  gs_cluster_dots(v0, l2, cnt, np, w, sh, sh.part[1], true);
+  cl.sync();
+  gs_cluster_gather(cl, sh.part[1], cnt + 1, sh.h2);
+  __syncthreads();
+  double s2 = sh.h2[cnt];
+  const bool refine = s2 < 0.5 * wn2;   // the same numbers in every CTA
+  if (refine) {
+    update(sh.h2);
+    gs_cluster_dots(v0, l2, cnt, np, w, sh, sh.part[2], false);
+    cl.sync();
+    gs_cluster_gather(cl, sh.part[2], 1, sh.h2 + 258);
+    __syncthreads();
+    s2 = sh.h2[258];
+  }
+  if (t == 0) {
+    const double nrm = sqrt(s2);
+    sh.scale = (nrm > 0.0) ? 1.0 / nrm : 0.0;
+  }
+  __syncthreads();
+  if (t < kGsWorkers) {
+    const double sc = sh.scale;
+    using T2 = typename Vec2<T>::type;
+    double2* vn = reinterpret_cast<double2*>(V + (size_t)(j + 1) * k.ld) + p0;
+#pragma unroll
+    for (int u = 0; u < kGsPairs; ++u) {
+      const int r = t + kGsWorkers * u;
+      if (r >= np) break;
+      double2 x = w[u];
+      x.x *= sc;
+      x.y *= sc;
+      vn[r] = x;
+      T2 o;
+      o.x = (T)x.x;
+      o.y = (T)x.y;
+      reinterpret_cast<T2*>(vin)[p0 + r] = o;
+    }
+  }
+  if (rank == 0) {
+    if (t == 0) {
+      k.ctl->refine = refine ? 1 : 0;
+      if (refine) k.ctl->refines += 1;
+    }
+    ArnoldiIn a = in;
+    if (t <= j) a.h1 = sh.h1[t];
+    arnoldi_finish(k, ash, a, j, refine ? sh.h2 : nullptr, s2);
+  }
+  cl.sync();   // no CTA leaves while another may still read its sums
 }
 
 // start of a cycle: beta = ||w|| with w = b - A x already formed
@@ -2111,13 +2316,57 @@ static void orthogonalise_launch(Problem& P, Prec<T>& pr, const KrylovArgs& k, c
   launch(k_basis<T>, nblk(P.n / 2, 256), 256, 0, s, (int)(P.n / 2), P.V, P.n, P.w, pr.vin, P.ctl);
 }
 
+template <class T>
+static cudaLaunchConfig_t gs_cluster_config(cudaLaunchAttribute* at, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kGsCluster);
+  cfg.blockDim = dim3(kRedThreads);
+  cfg.stream = s;
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = kGsCluster;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+// Whether the problem's orthogonalisation runs as one cluster: its rows fit, and
+// the device schedules a cluster of this (non-portable) size.  At 16 384 unknowns
+// the cluster's FP64 work has grown to what the separate launches cost.
+template <class T>
+static bool gs_cluster_fits(size_t n) {
+  if (n > (size_t)kGsCluster * kGsClusterRows) return false;
+  if (cudaFuncSetAttribute(k_gs_cluster<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  cudaLaunchAttribute at[1];
+  cudaLaunchConfig_t cfg = gs_cluster_config<T>(at, nullptr);
+  int num = 0;
+  if (cudaOccupancyMaxActiveClusters(&num, k_gs_cluster<T>, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return num > 0;
+}
+
+template <class T>
+static void gs_cluster_launch(Problem& P, Prec<T>& pr, const KrylovArgs& k, cudaStream_t s) {
+  cudaLaunchAttribute at[1];
+  const cudaLaunchConfig_t cfg = gs_cluster_config<T>(at, s);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_gs_cluster<T>, k, P.V, pr.vin);
+  if (e != cudaSuccess) throw CudaError(e, "cudaLaunchKernelEx (cluster orthogonalisation)");
+}
+
 // One Arnoldi iteration; pr.vin holds v_j on entry (k_basis of the previous
 // iteration or of the cycle's start wrote it).
 template <class T>
 static void iteration_launch(Problem& P, Prec<T>& pr, const KrylovArgs& k, cudaStream_t s) {
   precond_launch(P, pr, s);
   full_launch<T, double>(pr, pr.zw, P.w, nullptr, 1.0, 0.0, (T*)P.Z, P.n, P.ctl, s);
-  if (k.chunk == kChunkSmall) orthogonalise_launch<kChunkSmall>(P, pr, k, s);
+  if (P.gs_cluster) gs_cluster_launch<T>(P, pr, k, s);
+  else if (k.chunk == kChunkSmall) orthogonalise_launch<kChunkSmall>(P, pr, k, s);
   else orthogonalise_launch<kChunkLarge>(P, pr, k, s);
 }
 
@@ -2236,6 +2485,7 @@ static void build_graphs(Problem& P) {
   }
   CK(cudaStreamEndCapture(s, &P.gr_begin));
   CK(cudaGraphInstantiate(&P.g_begin, P.gr_begin, 0));
+  P.gs_cluster = P.prm.precision == 1 ? gs_cluster_fits<float>(P.n) : gs_cluster_fits<double>(P.n);
   // cycle
   const char* hl = getenv("FSI_HOST_LOOP");
   P.host_loop = hl && hl[0] == '1';
