@@ -88,12 +88,15 @@ constexpr int mf_pres_blk(int v, int y, int x) { return kMfPresVar * v + kMfPres
 // one global round trip, the barriers between its phases), not the work of
 // the overlaps the tiles repeat: on the 128 x 128 cavity, tiles shrunk to
 // keep 256 CTAs on every level measured slower (9.8 against 10.7 steps/s)
-// than one tile size for all levels.  From 512 cells on, the larger tiles
-// repeat less of their neighbours' work.  Up to 32 cells a velocity level takes
-// 4-node tiles: 64 CTAs of 384 threads instead of 16 of 512, down 3.35 -> 3.0 us,
+// than one tile size for all levels.  Where there are enough tiles to fill the
+// chip, larger ones repeat less of their neighbours' work: velocity levels above
+// 128 cells take 16-node tiles (256 cells, down / residual down / up: 14.3 / 24.0 /
+// 12.5 -> 9.9 / 16.1 / 8.4 us; 160 cells 7.2 / 12.9 / 6.2 -> 6.5 / 9.9 / 5.1),
+// pressure levels 8-cell tiles from 512 cells on (on 256 they are slower, 8.2 ->
+// 10.2 us).  Up to 32 cells a velocity level takes 4-node tiles: 64 CTAs of 384 threads instead of 16 of 512, down 3.35 -> 3.0 us,
 // up 3.3 -> 2.9 us on 32 cells (but 3.4 -> 5.8 us on 64, where they do not all fit
 // beside their four times repeated overlap).
-__host__ __device__ __forceinline__ int mf_tile_u(int N) { return N >= 512 ? 16 : (N > 32 ? 8 : 4); }
+__host__ __device__ __forceinline__ int mf_tile_u(int N) { return N > 128 ? 16 : (N > 32 ? 8 : 4); }
 __host__ __device__ __forceinline__ int mf_tile_p(int N) { return N >= 512 ? 8 : 4; }
 // Threads of a velocity launch.  A launch's time on these grids is one CTA's
 // chain of phases, and the threads' share of a phase sets it.  The stencil
@@ -137,6 +140,14 @@ inline void mf_with_tile_p(int N, F&& f) {
     case 2: f(std::integral_constant<int, 2>()); break;
     default: f(std::integral_constant<int, 1>()); break;
   }
+}
+
+// Call f(integral_constant<CTAs per SM>) for a pressure launch (see the kernels).
+template <bool UP, class F>
+inline void mf_with_minb_p(int N, F&& f) {
+  if (N <= 128) f(std::integral_constant<int, 1>());
+  else if (UP && N < 512) f(std::integral_constant<int, 8>());
+  else f(std::integral_constant<int, 6>());
 }
 
 template <class T>
@@ -1184,24 +1195,24 @@ __host__ __device__ void mfp_up_body(const MfPresArgs<T>& a, const MfCta& cta) {
 // The kernels: one CTA per tile, NT threads.
 // MINB: CTAs per SM the registers must leave room for.  Velocity: two, since the
 // 128-cell level has 256 CTAs for 152 SMs (one per SM cost 4.9 -> 6.7 us there).
-#define FSI_MF_BOUNDS_V __launch_bounds__(NT, TILE >= 8 ? 2 : 1)
-#define FSI_MF_BOUNDS_P __launch_bounds__(NT)
-#define FSI_MF_KERNEL(name, body, Args, BOUNDS)                                              \
-  template <class T, int TILE, int K, int NT>                                                \
-  __global__ void BOUNDS name(const __grid_constant__ Args<T> a) {            \
+// Pressure: one up to 128 cells, where every CTA has an SM's registers to itself
+// anyway (residual down on 128 cells 4.1 -> 3.6 us), above it six, eight for the
+// up launch of the 4-cell tiles (at one, 256 cells took 8.2 -> 10.4 and 5.3 -> 8.2 us).
+constexpr int mf_minb_u(int tc) { return tc >= 8 ? 2 : 1; }
+#define FSI_MF_KERNEL(name, body, Args)                                                      \
+  template <class T, int TILE, int K, int NT, int MINB>                                      \
+  __global__ void __launch_bounds__(NT, MINB) name(const __grid_constant__ Args<T> a) {            \
     asm volatile("griddepcontrol.wait;" ::: "memory");                                       \
     extern __shared__ __align__(16) unsigned char mf_smem[];                                 \
     const MfCta c{(int)blockIdx.x, (int)blockIdx.y, (int)threadIdx.x, (int)blockDim.x, NT,   \
                   mf_smem};                                                                  \
     body<T, TILE, K>(a, c);                                                                  \
   }
-FSI_MF_KERNEL(k_mfu_down, mfu_down_body, MfVelArgs, FSI_MF_BOUNDS_V)
-FSI_MF_KERNEL(k_mfu_up, mfu_up_body, MfVelArgs, FSI_MF_BOUNDS_V)
-FSI_MF_KERNEL(k_mfp_down, mfp_down_body, MfPresArgs, FSI_MF_BOUNDS_P)
-FSI_MF_KERNEL(k_mfp_up, mfp_up_body, MfPresArgs, FSI_MF_BOUNDS_P)
+FSI_MF_KERNEL(k_mfu_down, mfu_down_body, MfVelArgs)
+FSI_MF_KERNEL(k_mfu_up, mfu_up_body, MfVelArgs)
+FSI_MF_KERNEL(k_mfp_down, mfp_down_body, MfPresArgs)
+FSI_MF_KERNEL(k_mfp_up, mfp_up_body, MfPresArgs)
 #undef FSI_MF_KERNEL
-#undef FSI_MF_BOUNDS_V
-#undef FSI_MF_BOUNDS_P
 #endif
 
 // shared memory of one launch (bytes) for tile tc (velocity: coarse lattice

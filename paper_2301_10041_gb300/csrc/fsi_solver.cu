@@ -618,9 +618,9 @@ static void select_mf(MG<T>& mg, const HostSetup& hs, int mg_fused, bool count_o
           mf_with_degree(K, [&](auto kc) {
             constexpr int TC = decltype(tc)::value, KD = decltype(kc)::value;
             constexpr int ND = mf_threads_ud(TC), NU = mf_threads_uu(TC);
-            CK(cudaFuncSetAttribute(k_mfu_down<float, TC, KD, ND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            CK(cudaFuncSetAttribute(k_mfu_down<float, TC, KD, ND, mf_minb_u(TC)>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)mfu_down_smem<float>(TC, KD)));
-            CK(cudaFuncSetAttribute(k_mfu_up<float, TC, KD, NU>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            CK(cudaFuncSetAttribute(k_mfu_up<float, TC, KD, NU, mf_minb_u(TC)>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)mfu_up_smem<float>(TC, KD)));
           });
       };
@@ -628,10 +628,18 @@ static void select_mf(MG<T>& mg, const HostSetup& hs, int mg_fused, bool count_o
         for (int K = 1; K <= kMfMaxDeg; ++K)
           mf_with_degree(K, [&](auto kc) {
             constexpr int TP = decltype(tp)::value, KD = decltype(kc)::value, NT = mf_threads_p(TP);
-            CK(cudaFuncSetAttribute(k_mfp_down<float, TP, KD, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)mfp_down_smem<float>(TP, KD)));
-            CK(cudaFuncSetAttribute(k_mfp_up<float, TP, KD, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)mfp_up_smem<float>(TP, KD)));
+            for (int n : {128, 256, 512}) {
+              mf_with_minb_p<false>(n, [&](auto mb) {
+                CK(cudaFuncSetAttribute(k_mfp_down<float, TP, KD, NT, decltype(mb)::value>,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)mfp_down_smem<float>(TP, KD)));
+              });
+              mf_with_minb_p<true>(n, [&](auto mb) {
+                CK(cudaFuncSetAttribute(k_mfp_up<float, TP, KD, NT, decltype(mb)::value>,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)mfp_up_smem<float>(TP, KD)));
+              });
+            }
           });
       };
       for (int N : {16, 64, 128, 512}) mf_with_tile_u(N, vel);   // every tile the maps choose
@@ -682,7 +690,9 @@ static void mf_down_launch(MG<T>& mg, int l, const T* b, cudaStream_t s, const M
       mf_with_degree(K, [&](auto kc) {
         constexpr int TP = decltype(tp)::value, KD = decltype(kc)::value, NT = mf_threads_p(TP);
         const unsigned g = nblk(N / 2, TP);
-        launch(k_mfp_down<T, TP, KD, NT>, dim3(g, g), NT, mfp_down_smem<T>(TP, KD), s, a);
+        mf_with_minb_p<false>(N, [&](auto mb) {
+          launch(k_mfp_down<T, TP, KD, NT, decltype(mb)::value>, dim3(g, g), NT, mfp_down_smem<T>(TP, KD), s, a);
+        });
       });
     });
   } else {
@@ -693,7 +703,7 @@ static void mf_down_launch(MG<T>& mg, int l, const T* b, cudaStream_t s, const M
       mf_with_degree(K, [&](auto kc) {
         constexpr int TC = decltype(tc)::value, KD = decltype(kc)::value, NT = mf_threads_ud(TC);
         const unsigned g = nblk(N, TC);
-        launch(k_mfu_down<T, TC, KD, NT>, dim3(g, g), NT, mfu_down_smem<T>(TC, KD), s, a);
+        launch(k_mfu_down<T, TC, KD, NT, mf_minb_u(TC)>, dim3(g, g), NT, mfu_down_smem<T>(TC, KD), s, a);
       });
     });
   }
@@ -715,7 +725,9 @@ static void mf_up_launch(MG<T>& mg, int l, const T* b, const T* xc, T* dst, cons
       mf_with_degree(K, [&](auto kc) {
         constexpr int TP = decltype(tp)::value, KD = decltype(kc)::value, NT = mf_threads_p(TP);
         const unsigned g = nblk(N, 2 * TP);
-        launch(k_mfp_up<T, TP, KD, NT>, dim3(g, g), NT, mfp_up_smem<T>(TP, KD), s, a);
+        mf_with_minb_p<true>(N, [&](auto mb) {
+          launch(k_mfp_up<T, TP, KD, NT, decltype(mb)::value>, dim3(g, g), NT, mfp_up_smem<T>(TP, KD), s, a);
+        });
       });
     });
   } else {
@@ -727,7 +739,7 @@ static void mf_up_launch(MG<T>& mg, int l, const T* b, const T* xc, T* dst, cons
       mf_with_degree(K, [&](auto kc) {
         constexpr int TC = decltype(tc)::value, KD = decltype(kc)::value, NT = mf_threads_uu(TC);
         const unsigned g = nblk(2 * N, 2 * TC);
-        launch(k_mfu_up<T, TC, KD, NT>, dim3(g, g), NT, mfu_up_smem<T>(TC, KD), s, a);
+        launch(k_mfu_up<T, TC, KD, NT, mf_minb_u(TC)>, dim3(g, g), NT, mfu_up_smem<T>(TC, KD), s, a);
       });
     });
   }
