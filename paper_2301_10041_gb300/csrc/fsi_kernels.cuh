@@ -575,8 +575,6 @@ __global__ void __launch_bounds__(128) k_cf_apply(int nS, int cap, const int* __
 }
 
 // ------------------------------------------------------------ small dense
-// y = A x for a dense row-major n x n matrix (coarsest multigrid level):
-// one warp per row, lanes over the columns, 8 rows per CTA
 // 16-byte vector of T
 template <class T>
 struct Vec16;
@@ -629,6 +627,128 @@ __global__ void k_dense_mv(int n, int ld, const T* __restrict__ A, const T* __re
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
   if (lane == 0) y[i] = s;
+}
+
+// The dense inverse G of the coarsest level through its mirror symmetry.  The
+// square grid, its walls and the level operators are unchanged by the mirrors
+// in x = 1/2 and y = 1/2 (a mirrored vector flips its normal component, a cell's
+// linear coefficients their sign), so G maps each of the four symmetry classes
+// (even or odd in x, even or odd in y) to itself.  A class is given by its values
+// on one quarter of the grid: R representatives (r), with images r, mx r, my r,
+// mxy r and signs sx, sy.  With t_s[q] the sum of the images of q, signed by class s,
+// the class's part of G b at r is sum_q G_s[r][q] t_s[q], with
+//   G_s[r][q] = 1/4 sum over the distinct images j of q, signed by s, of G[r][j],
+// and the result at an image of r is the signed sum over the four classes.  So a
+// quarter of the entries and of the multiply-adds are left: in FP64 these are
+// the bound (64 cycles per warp instruction), in FP32 the read from L2.
+struct SymMap {
+  int R = 0;                    // representatives
+  const int4* img = nullptr;    // images (r, mx r, my r, mxy r) of each
+  const int* sgn = nullptr;     // bit 0: sx = -1, bit 1: sy = -1
+};
+
+// sum over the images of v, signed by the four classes: t[2 b + a], class a odd
+// under the mirror in x when a = 1, b under the one in y
+template <class T>
+__device__ __forceinline__ void sym_split(T v0, T v1, T v2, T v3, int sgn, T t[4]) {
+  if (sgn & 1) { v1 = -v1; v3 = -v3; }
+  if (sgn & 2) { v2 = -v2; v3 = -v3; }
+  const T e0 = v0 + v1, o0 = v0 - v1, e1 = v2 + v3, o1 = v2 - v3;
+  t[0] = e0 + e1;
+  t[1] = o0 + o1;
+  t[2] = e0 - e1;
+  t[3] = o0 - o1;
+}
+
+// A CTA takes blockDim / 128 representatives, four warps each (one per class):
+// all of b into its class sums in shared memory, the rows' dots, the images.
+// Rows hold ld >= R entries (16-byte multiples, zero padding).
+template <class T>
+__global__ void __launch_bounds__(512) k_dense_sym(SymMap m, int ld, const T* __restrict__ G, const T* __restrict__ x,
+                                                   T* __restrict__ y) {
+  using V = typename Vec16<T>::type;
+  constexpr int W = 16 / (int)sizeof(T), U = 4;
+  extern __shared__ __align__(16) unsigned char sym_smem[];
+  T* ts = reinterpret_cast<T*>(sym_smem);          // 4 x ld
+  __shared__ T part[16];
+  pdl_begin();
+  for (int q = threadIdx.x; q < ld; q += blockDim.x) {
+    T t[4] = {0, 0, 0, 0};
+    if (q < m.R) {
+      const int4 j = m.img[q];
+      sym_split<T>(x[j.x], x[j.y], x[j.z], x[j.w], m.sgn[q], t);
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) ts[c * ld + q] = t[c];
+  }
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, cls = w & 3;
+  const int r = blockIdx.x * (blockDim.x >> 7) + (w >> 2);
+  const bool live = r < m.R;
+  const V* __restrict__ g = reinterpret_cast<const V*>(G + ((size_t)cls * m.R + (live ? r : 0)) * ld);
+  const V* tv = reinterpret_cast<const V*>(ts + cls * ld);
+  const int nv = ld / W;
+  V pre[U];   // the row's first vectors, in flight across the barrier
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+    if (lane + 32 * u < nv) pre[u] = __ldg(g + lane + 32 * u);
+  __syncthreads();
+  T acc[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) acc[u] = (lane + 32 * u < nv) ? Vec16<T>::dot(pre[u], tv[lane + 32 * u], (T)0) : (T)0;
+  for (int j0 = lane + 32 * U; j0 < nv; j0 += 32 * U) {
+    V av[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (j0 + 32 * u < nv) av[u] = __ldg(g + j0 + 32 * u);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (j0 + 32 * u < nv) acc[u] = Vec16<T>::dot(av[u], tv[j0 + 32 * u], acc[u]);
+  }
+  T s = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if (lane == 0) part[w] = s;
+  __syncthreads();
+  if (threadIdx.x < (blockDim.x >> 5) && (threadIdx.x & 3) == 0) {
+    const int rr = blockIdx.x * (blockDim.x >> 7) + (threadIdx.x >> 2);
+    if (rr < m.R) {
+      const T* p = part + threadIdx.x;
+      const int4 j = m.img[rr];
+      T v[4];   // v[image] = sum over the classes, signed: the same butterfly
+      sym_split<T>(p[0], p[1], p[2], p[3], 0, v);
+      const int sg = m.sgn[rr];
+      y[j.x] = v[0];
+      y[j.y] = (sg & 1) ? -v[1] : v[1];
+      y[j.z] = (sg & 2) ? -v[2] : v[2];
+      y[j.w] = ((sg ^ (sg >> 1)) & 1) ? -v[3] : v[3];
+    }
+  }
+}
+
+// the class matrices from the full inverse (rows of ldi entries); a row or
+// column whose representative lies on a mirror line and is odd there is zero
+template <class T>
+__global__ void k_sym_build(SymMap m, int ld, const double* __restrict__ G, int ldi, T* __restrict__ out) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y, cls = blockIdx.z;
+  if (q >= ld) return;
+  double v = 0;
+  if (q < m.R) {
+    const int4 i = m.img[r], j = m.img[q];
+    const int sr = m.sgn[r], sq = m.sgn[q];
+    const double ca = (cls & 1) ? -1.0 : 1.0, cb = (cls & 2) ? -1.0 : 1.0;
+    const double ax = ca * ((sq & 1) ? -1.0 : 1.0), ay = cb * ((sq & 2) ? -1.0 : 1.0);
+    const bool zr = (i.y == i.x && ca * ((sr & 1) ? -1.0 : 1.0) < 0) || (i.z == i.x && cb * ((sr & 2) ? -1.0 : 1.0) < 0);
+    const bool zq = (j.y == j.x && ax < 0) || (j.z == j.x && ay < 0);
+    if (!zr && !zq) {
+      const double* g = G + (size_t)i.x * ldi;
+      v = g[j.x];
+      if (j.y != j.x) v += ax * g[j.y];
+      if (j.z != j.x) v += ay * g[j.z];
+      if (j.y != j.x && j.z != j.x) v += ax * ay * g[j.w];
+      v *= 0.25;
+    }
+  }
+  out[((size_t)cls * m.R + r) * ld + q] = (T)v;
 }
 
 // ------------------------------------------------ coarsest-level inverse

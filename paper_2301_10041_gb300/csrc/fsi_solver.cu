@@ -337,6 +337,9 @@ struct MG {
   T* coarse_inv = nullptr;   // dense inverse of the coarsest level, rows of coarse_ld entries
   int coarse_n = 0;
   int coarse_ld = 0;         // coarse_n rounded up to 16 bytes (the row padding is zero)
+  SymMap sym;                // its mirror images, and the class matrices (k_dense_sym)
+  T* sym_inv = nullptr;      // 4 x sym.R rows of sym_ld entries
+  int sym_ld = 0;
   int degree = 2;
   bool pressure = false;
   ClusterMG<T> cl;
@@ -370,6 +373,33 @@ static int dense_ld(int n) {
   return (n + w - 1) / w * w;
 }
 
+// Representatives of the coarsest level under the two mirrors (SymMap): scalar
+// unknown i at mirrored positions.  Velocity: 2 node + component, the component
+// along the mirror's normal flips; pressure: 3 cell + coefficient, the linear
+// coefficient in the mirrored direction flips.
+static void sym_images(int N, bool pressure, std::vector<int4>& img, std::vector<int>& sgn) {
+  const VNum vn(pressure ? 0 : N);
+  const int half = pressure ? (N + 1) / 2 : N, lo = pressure ? 0 : 1, nk = pressure ? 3 : 2;
+  auto id = [&](int x, int y, int k) { return pressure ? 3 * (y * N + x) + k : 2 * vn.id(x, y) + k; };
+  const int mir = pressure ? N - 1 : 2 * N;
+  for (int y = lo; y < lo + half; ++y)
+    for (int x = lo; x < lo + half; ++x)
+      for (int k = 0; k < nk; ++k) {
+        int4 j;
+        j.x = id(x, y, k);
+        j.y = id(mir - x, y, k);
+        j.z = id(x, mir - y, k);
+        j.w = id(mir - x, mir - y, k);
+        img.push_back(j);
+        sgn.push_back(pressure ? (k == 1 ? 1 : 0) | (k == 2 ? 2 : 0) : (k == 0 ? 1 : 2));
+      }
+}
+
+constexpr int kSymMinF32 = 1500;   // coarsest unknowns from which the FP32 product goes by classes
+constexpr int kSymThreadsF32 = 256, kSymThreadsF64 = 512;   // two and four representatives per CTA
+template <class T>
+constexpr int sym_threads() { return sizeof(T) == 8 ? kSymThreadsF64 : kSymThreadsF32; }
+
 // The coarsest level's dense inverse: the FP64 hierarchy inverts the
 // assembled matrix in place; the FP32 one rounds the FP64 inverse (inv64,
 // rows of ld64 entries).  The FP64 hierarchy is built first.
@@ -393,6 +423,32 @@ static void build_coarse_inverse(Arena& ar, const HostSetup& hs, bool pressure, 
     if (!inv64) throw std::logic_error("the FP64 coarse inverse is built first");
     k_dense_round<T><<<dim3((ld + 255) / 256, n), 256, 0, s>>>(n, inv64, ld64, mg.coarse_inv, ld);
     CK(cudaGetLastError());
+  }
+  // the class matrices of the dense product, from the FP64 inverse.  In FP32
+  // they pay from some 1500 unknowns on (1922: 2.93 -> 2.61 us, but 1058: 2.19 ->
+  // 2.38, 768: 1.69 -> 1.90, the class sums outweighing the shorter read); in FP64
+  // the multiply-adds saved always do (1922: 11.7 -> 7.3 us, 768: 5.6 -> 4.9).
+  if (sizeof(T) == 8 || n >= kSymMinF32) {
+    std::vector<int4> img;
+    std::vector<int> sgn;
+    sym_images(mg.lv.back().N, pressure, img, sgn);
+    mg.sym.R = (int)img.size();
+    mg.sym.img = ar.upload(img);
+    mg.sym.sgn = ar.upload(sgn);
+    mg.sym_ld = dense_ld<T>(mg.sym.R);
+    mg.sym_inv = ar.alloc<T>(4 * (size_t)mg.sym.R * mg.sym_ld);
+    if (!ar.count_only) {
+      const double* full = inv64;
+      int fld = ld64;
+      if constexpr (std::is_same<T, double>::value) {
+        full = mg.coarse_inv;
+        fld = ld;
+      }
+      k_sym_build<T><<<dim3(nblk(mg.sym_ld, 128), mg.sym.R, 4), 128, 0, s>>>(mg.sym, mg.sym_ld, full, fld, mg.sym_inv);
+      CK(cudaGetLastError());
+      if (4 * (size_t)mg.sym_ld * sizeof(T) > 48 * 1024)
+        CK(cudaFuncSetAttribute(k_dense_sym<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    }
   }
   // the coarsest right-hand side, padded to ld with zeros, for the dense product
   MGLevel<T>& C = mg.lv.back();
@@ -813,9 +869,9 @@ static MfWork vcycle_work(const HostSetup& hs, const MG<T>& mg, bool pressure) {
     w.bytes += (2 * K + 1) * (a_bytes + 4.0 * n * ts) + t_bytes;
     w.flops += (2 * K + 1) * a_flops + 2.0 * (R.nnzb() + Pm.nnzb()) * (R.kron ? R.BR : R.BR * R.BC);
   }
-  const double nc = mg.coarse_n;
-  w.bytes += nc * mg.coarse_ld * ts + 2.0 * nc * ts;
-  w.flops += 2.0 * nc * nc;
+  const double nc = mg.coarse_n, R = mg.sym.R;   // the inverse, or its four class matrices, once
+  w.bytes += (R > 0 ? 4.0 * R * R : nc * mg.coarse_ld) * ts + 2.0 * nc * ts;
+  w.flops += R > 0 ? 8.0 * R * R : 2.0 * nc * nc;
   return w;
 }
 
@@ -849,8 +905,15 @@ static T* vcycle(MG<T>& mg, int l, cudaStream_t s, T* out, const SpmvArgs<T>* fi
     return dst;
   }
   if (l == last) {
-    launch(k_dense_mv<T>, nblk(mg.coarse_n, 8), 256, 0, s, mg.coarse_n, mg.coarse_ld, (const T*)mg.coarse_inv,
-           (const T*)L.b, out ? out : L.x);
+    if constexpr (sizeof(T) == 4) {
+      if (mg.sym.R == 0) {
+        launch(k_dense_mv<T>, nblk(mg.coarse_n, 8), 256, 0, s, mg.coarse_n, mg.coarse_ld, (const T*)mg.coarse_inv,
+               (const T*)L.b, out ? out : L.x);
+        return out ? out : L.x;
+      }
+    }
+    launch(k_dense_sym<T>, nblk(mg.sym.R, sym_threads<T>() / 128), sym_threads<T>(),
+           4 * (size_t)mg.sym_ld * sizeof(T), s, mg.sym, mg.sym_ld, (const T*)mg.sym_inv, (const T*)L.b, out ? out : L.x);
     return out ? out : L.x;
   }
   T* xc = L.x;
@@ -1038,7 +1101,8 @@ static void setup_solid_patches(Arena& ar, const HostSetup& hs, const double* re
   constexpr bool f64 = std::is_same<T, double>::value;
   constexpr int NT = sc_threads<T>();
   SolidPatchHost h;
-  if (!build_solid_patches(hs.Cs, ref_xy, pr.cs_k - 1, f64, NT, h)) {
+  if (!build_solid_patches(hs.Cs, ref_xy, pr.cs_k - 1, f64, NT, h) ||
+      4 * sizeof(T) * (size_t)h.max_loc > kClSmemCap) {   // an outer layer too long for the iterate's two copies
     if (ar.count_only) {
       const SolidPlan pl = plan_solid_patches(hs.Cs.nrows, pr.cs_k - 1, f64, 2 * NT);
       const double r = std::sqrt((double)hs.Cs.nrows / std::max(1, pl.np)) + 2.0 * pl.steps;
