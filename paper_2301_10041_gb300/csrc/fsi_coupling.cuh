@@ -267,15 +267,17 @@ __device__ __forceinline__ int sh_clip(const double (*in)[2], int n, double (*ou
   return m;
 }
 
-// Contribution of one (mapped solid triangle, fluid cell) pair to row l:
-// acc[3 bb + aa] = (|E| / |X(E)|) * integral over X(E) cut by the cell of
-// lambda_a(x) phi_{aa,bb}(x), with the piece split from its first vertex into
-// triangles and Radon's degree-5 rule on each (the integrand is linear times
-// biquadratic).
-__device__ __forceinline__ void exact_pair(const double (*P)[2], double det, double scale, int a, int cx, int cy,
+// Contributions of one (mapped solid triangle, fluid cell) pair to the rows of
+// vertices a0 .. a0 + NA - 1: acc[9 a + 3 bb + aa] = (|E| / |X(E)|) * integral over
+// X(E) cut by the cell of lambda_a(x) phi_{aa,bb}(x), with the piece split from its
+// first vertex into triangles and Radon's degree-5 rule on each (the integrand is
+// linear times biquadratic).  The barycentric and cell coordinates are affine, so
+// they are formed at the piece's vertices and combined at the rule's points.
+template <int NA>
+__device__ __forceinline__ void exact_pair(const double (*P)[2], double det, double scale, int a0, int cx, int cy,
                                            int N, double* acc) {
 #pragma unroll
-  for (int k = 0; k < 9; ++k) acc[k] = 0.0;
+  for (int k = 0; k < 9 * NA; ++k) acc[k] = 0.0;
   const double h = 1.0 / (double)N;
   double b0[kClipMax][2], b1[kClipMax][2];
   b0[0][0] = P[0][0]; b0[0][1] = P[0][1];
@@ -291,39 +293,119 @@ __device__ __forceinline__ void exact_pair(const double (*P)[2], double det, dou
   const double d2x = P[2][0] - P[0][0], d2y = P[2][1] - P[0][1];
   const double idet = 1.0 / det;       // one division per pair: the FP64 pipe is the bound
   const double fN = (double)N;
+  // (xi, eta, lambda_1, lambda_2) of a vertex of the piece
+  auto coords = [&](const double* v, double o[4]) {
+    const double rx = v[0] - P[0][0], ry = v[1] - P[0][1];
+    o[0] = v[0] * fN - cx;
+    o[1] = v[1] * fN - cy;
+    o[2] = (rx * d2y - ry * d2x) * idet;
+    o[3] = (d1x * ry - d1y * rx) * idet;
+  };
+  double c0[4], c1[4], c2[4];
+  coords(b0[0], c0);
+  coords(b0[1], c2);
   for (int i = 1; i + 1 < n; ++i) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) c1[k] = c2[k];
+    coords(b0[i + 1], c2);
     const double e1x = b0[i][0] - b0[0][0], e1y = b0[i][1] - b0[0][1];
     const double e2x = b0[i + 1][0] - b0[0][0], e2y = b0[i + 1][1] - b0[0][1];
     const double asub = 0.5 * fabs(e1x * e2y - e1y * e2x);
     if (asub == 0.0) continue;
     for (int q = 0; q < 7; ++q) {
-      const double xq = c_radon_lam[q][0] * b0[0][0] + c_radon_lam[q][1] * b0[i][0] + c_radon_lam[q][2] * b0[i + 1][0];
-      const double yq = c_radon_lam[q][0] * b0[0][1] + c_radon_lam[q][1] * b0[i][1] + c_radon_lam[q][2] * b0[i + 1][1];
-      const double rx = xq - P[0][0], ry = yq - P[0][1];
-      const double l1 = (rx * d2y - ry * d2x) * idet;
-      const double l2 = (d1x * ry - d1y * rx) * idet;
-      const double la = (a == 0) ? 1.0 - l1 - l2 : (a == 1 ? l1 : l2);
-      const double xi = xq * fN - cx, eta = yq * fN - cy;
-      const double wq = asub * c_radon_w[q] * la;
+      const double m0 = c_radon_lam[q][0], m1 = c_radon_lam[q][1], m2 = c_radon_lam[q][2];
+      double v[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[k] = m0 * c0[k] + m1 * c1[k] + m2 * c2[k];
+      const double wq = asub * c_radon_w[q];
       double bx[3], by[3];
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
-        bx[j] = q2b(j, xi);
-        by[j] = q2b(j, eta);
+        bx[j] = q2b(j, v[0]);
+        by[j] = q2b(j, v[1]);
       }
 #pragma unroll
-      for (int bb = 0; bb < 3; ++bb)
+      for (int t = 0; t < NA; ++t) {
+        const int a = a0 + t;
+        const double la = wq * ((a == 0) ? 1.0 - v[2] - v[3] : (a == 1 ? v[2] : v[3]));
 #pragma unroll
-        for (int aa = 0; aa < 3; ++aa) acc[3 * bb + aa] += wq * bx[aa] * by[bb];
+        for (int aa = 0; aa < 3; ++aa) {
+          const double w = la * bx[aa];
+#pragma unroll
+          for (int bb = 0; bb < 3; ++bb) acc[9 * t + 3 * bb + aa] += w * by[bb];
+        }
+      }
     }
   }
 #pragma unroll
-  for (int k = 0; k < 9; ++k) acc[k] *= scale;
+  for (int k = 0; k < 9 * NA; ++k) acc[k] *= scale;
+}
+
+// the cells of a triangle's bounding box; false when a vertex lies outside [0,1]^2
+__device__ __forceinline__ bool exact_box(const double (*P)[2], int N, int& cx0, int& cy0, int& bw, int& cnt) {
+  double lo[2] = {2.0, 2.0}, hi[2] = {-1.0, -1.0};
+  for (int v = 0; v < 3; ++v)
+    for (int c = 0; c < 2; ++c) {
+      const double xc = P[v][c];
+      if (!(xc >= 0.0 && xc <= 1.0)) return false;
+      lo[c] = fmin(lo[c], xc);
+      hi[c] = fmax(hi[c], xc);
+    }
+  cx0 = min((int)floor(lo[0] * N), N - 1);
+  cy0 = min((int)floor(lo[1] * N), N - 1);
+  const int cx1 = min((int)floor(hi[0] * N), N - 1), cy1 = min((int)floor(hi[1] * N), N - 1);
+  bw = cx1 - cx0 + 1;
+  cnt = bw * (cy1 - cy0 + 1);
+  return true;
+}
+
+__device__ __forceinline__ void exact_load(const int* __restrict__ tris, const double* __restrict__ X, int t,
+                                           double (*P)[2]) {
+#pragma unroll
+  for (int v = 0; v < 3; ++v) {
+    const int node = tris[3 * t + v];
+    P[v][0] = X[2 * node];
+    P[v][1] = X[2 * node + 1];
+  }
+}
+
+// The pairs of every triangle that overlaps at most kExactCells cells (a body
+// refined with the fluid grid has no other), for its three vertices at once: the
+// clip, the points and the basis of a pair serve three rows, which took them
+// three times over when each row formed its own.  Bound by the FP64 pipe, as the
+// rows were: assembly on 256 cells (63 654 triangles) 2.69 -> 1.23 ms, 0.27 ms on
+// 128 cells; the 55 MB of pairs (on 256 cells) are written and read once, 15 us at
+// the HBM rate.  Four cells, since a triangle no wider than a cell lies in a box of
+// at most 2 x 2; a larger one would leave most of a fixed-size slot unused.  pairs[(9 a + k) M + 4 t + s]:
+// entry k of vertex a for cell s of triangle t, M = 4 n_tris.
+constexpr int kExactCells = 4;
+__global__ void __launch_bounds__(128) k_exact_pairs(int n_tris, int N, const int* __restrict__ tris,
+                                                     const double* __restrict__ X, const double* __restrict__ area,
+                                                     double* __restrict__ pairs) {
+  pdl_begin();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, t = i / kExactCells, s = i - kExactCells * t;
+  if (t >= n_tris) return;
+  double P[3][2];
+  exact_load(tris, X, t, P);
+  int cx0, cy0, bw, cnt;
+  if (!exact_box(P, N, cx0, cy0, bw, cnt) || cnt > kExactCells || s >= cnt) return;
+  const double det = (P[1][0] - P[0][0]) * (P[2][1] - P[0][1]) - (P[1][1] - P[0][1]) * (P[2][0] - P[0][0]);
+  double acc[27];
+  if (det != 0.0) {
+    exact_pair<3>(P, det, area[t] / (0.5 * fabs(det)), 0, cx0 + s % bw, cy0 + s / bw, N, acc);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 27; ++k) acc[k] = 0.0;
+  }
+  const size_t M = (size_t)kExactCells * n_tris;
+#pragma unroll
+  for (int k = 0; k < 27; ++k) pairs[k * M + i] = acc[k];
 }
 
 // S4 with the paper's exact rule (Section 4): one warp per solid node l.
 // Every (triangle of l, fluid cell of the triangle's bounding box) pair is one
-// work item; the lanes take 32 items at a time, and their 9 contributions are
+// work item (read from k_exact_pairs, or formed here for a triangle over more than
+// kExactCells cells); the lanes take 32 items at a time, and their 9 contributions are
 // added to the row window in item order (no atomics, deterministic), then
 // compacted as in k_cf_rows.  A vertex outside [0,1]^2 raises
 // FLAG_OUT_OF_DOMAIN; more than 32 triangles at a node or a window above
@@ -332,7 +414,8 @@ __global__ void __launch_bounds__(32 * kCfWarps) k_cf_rows_exact(
     int nS, int N, const int* __restrict__ ntp, const int* __restrict__ nt, const int* __restrict__ tris,
     const double* __restrict__ X, const double* __restrict__ area, const int* __restrict__ l2n,
     const double* __restrict__ wall, int cap, int* __restrict__ len, int* __restrict__ col,
-    double* __restrict__ val, float* __restrict__ val32, double* __restrict__ lift, int* __restrict__ flags) {
+    double* __restrict__ val, float* __restrict__ val32, double* __restrict__ lift, int* __restrict__ flags,
+    const double* __restrict__ pairs, int n_tris) {
   pdl_begin();
   __shared__ double win[kCfWarps][kCfWindow];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -347,23 +430,10 @@ __global__ void __launch_bounds__(32 * kCfWarps) k_cf_rows_exact(
     const int e = nt[e0 + lane];
     t = e / 3;
     a = e - 3 * t;
-    double lo[2] = {2.0, 2.0}, hi[2] = {-1.0, -1.0};
-    for (int v = 0; v < 3; ++v) {
-      const int node = tris[3 * t + v];
-      for (int c = 0; c < 2; ++c) {
-        const double xc = X[2 * node + c];
-        if (!(xc >= 0.0 && xc <= 1.0)) outside = true;
-        lo[c] = fmin(lo[c], xc);
-        hi[c] = fmax(hi[c], xc);
-      }
-    }
-    if (!outside) {
-      cx0 = min((int)floor(lo[0] * N), N - 1);
-      cy0 = min((int)floor(lo[1] * N), N - 1);
-      const int cx1 = min((int)floor(hi[0] * N), N - 1), cy1 = min((int)floor(hi[1] * N), N - 1);
-      bw = cx1 - cx0 + 1;
-      cnt = bw * (cy1 - cy0 + 1);
-    }
+    double P[3][2];
+    exact_load(tris, X, t, P);
+    outside = !exact_box(P, N, cx0, cy0, bw, cnt);
+    if (outside) cx0 = cy0 = bw = cnt = 0;
   }
   const bool bad = __any_sync(0xffffffffu, outside);
   // window: union of the cell boxes
@@ -410,19 +480,24 @@ __global__ void __launch_bounds__(32 * kCfWarps) k_cf_rows_exact(
       const int tk = __shfl_sync(0xffffffffu, t, k), ak = __shfl_sync(0xffffffffu, a, k);
       const int bx0 = __shfl_sync(0xffffffffu, cx0, k), by0 = __shfl_sync(0xffffffffu, cy0, k);
       const int bwk = __shfl_sync(0xffffffffu, bw, k), ek = __shfl_sync(0xffffffffu, excl, k);
-      if (i < nitems) {
+      const int ck = __shfl_sync(0xffffffffu, cnt, k);
+      if (i < nitems && ck <= kExactCells) {
+        const int j = i - ek;
+        cx = bx0 + j % bwk;
+        cy = by0 + j / bwk;
+        const size_t M = (size_t)kExactCells * n_tris;
+        const double* __restrict__ p = pairs + 9 * (size_t)ak * M + (size_t)kExactCells * tk + j;
+#pragma unroll
+        for (int q = 0; q < 9; ++q) acc[q] = p[q * M];
+      } else if (i < nitems) {
         const int j = i - ek;
         cx = bx0 + j % bwk;
         cy = by0 + j / bwk;
         double P[3][2];
-        for (int v = 0; v < 3; ++v) {
-          const int node = tris[3 * tk + v];
-          P[v][0] = X[2 * node];
-          P[v][1] = X[2 * node + 1];
-        }
+        exact_load(tris, X, tk, P);
         const double det = (P[1][0] - P[0][0]) * (P[2][1] - P[0][1]) - (P[1][1] - P[0][1]) * (P[2][0] - P[0][0]);
         if (det != 0.0) {
-          exact_pair(P, det, area[tk] / (0.5 * fabs(det)), ak, cx, cy, N, acc);
+          exact_pair<1>(P, det, area[tk] / (0.5 * fabs(det)), ak, cx, cy, N, acc);
         } else {
 #pragma unroll
           for (int q = 0; q < 9; ++q) acc[q] = 0.0;

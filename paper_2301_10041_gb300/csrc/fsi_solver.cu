@@ -1013,6 +1013,7 @@ struct Problem {
   int* l2n = nullptr; double* wall = nullptr;
   int* cell = nullptr; double* xi = nullptr; double* eta = nullptr;
   int cf_cap = 64;
+  double* pairs = nullptr;   // exact rule: contributions per (triangle, cell) pair (k_exact_pairs)
   // nonlinear solid: reference gradients of the P1 basis per triangle (3 x 2),
   // tangent blocks in the slots of the solid pair matrix (4 per slot)
   double* tgrad = nullptr;
@@ -2345,6 +2346,13 @@ static KrylovArgs krylov_args(Problem& P, cudaGraphConditionalHandle h) {
   return k;
 }
 
+// S4 by the exact rule: the pairs of small triangles, then the C_f rows.
+static void exact_rule_launch(Problem& P, cudaStream_t s) {
+  launch(k_exact_pairs, nblk((size_t)kExactCells * P.nTri, 128), 128, 0, s, P.nTri, P.N, P.tris, P.Xold, P.area, P.pairs);
+  launch(k_cf_rows_exact, nblk(P.nS, kCfWarps), 32 * kCfWarps, 0, s, P.nS, P.N, P.ntp, P.nt, P.tris, P.Xold, P.area,
+         P.l2n, P.wall, P.cf_cap, P.cf_len, P.cf_col, P.cf_val, P.cf_val32, P.cflift, &P.ctl->aflags, P.pairs, P.nTri);
+}
+
 // S2 + S4 by the point rule: locate the rule points, then the C_f rows.
 static void point_rule_launch(Problem& P, cudaStream_t s) {
   if (elem_nodes(P.prm) == 4) {
@@ -2363,8 +2371,7 @@ static void point_rule_launch(Problem& P, cudaStream_t s) {
 static void assemble_launch(Problem& P, cudaStream_t s) {
   CK(cudaMemsetAsync(&P.ctl->aflags, 0, sizeof(int), s));
   if (P.prm.coupling == 1) {  // the paper's exact rule: mesh intersection
-    launch(k_cf_rows_exact, nblk(P.nS, kCfWarps), 32 * kCfWarps, 0, s, P.nS, P.N, P.ntp, P.nt, P.tris, P.Xold, P.area,
-           P.l2n, P.wall, P.cf_cap, P.cf_len, P.cf_col, P.cf_val, P.cf_val32, P.cflift, &P.ctl->aflags);
+    exact_rule_launch(P, s);
   } else {                    // located points of the point rule
     point_rule_launch(P, s);
   }
@@ -2594,6 +2601,7 @@ static void allocate_problem(Problem& P, const double* ref_xy, const int* tris_h
   P.nt = ar.upload(hs.node_tri);
   P.l2n = ar.upload(hs.lattice_to_node);
   P.wall = ar.upload(hs.wall_u);
+  if (P.prm.coupling == 1) P.pairs = ar.alloc<double>(27 * (size_t)kExactCells * P.nTri);
   P.cell = ar.alloc<int>(P.nPts);
   P.xi = ar.alloc<double>(P.nPts);
   P.eta = ar.alloc<double>(P.nPts);
@@ -3360,8 +3368,7 @@ int fsi_time_kernel(fsi_problem* h, int which, int reps, double* avg_ms, double*
           *bytes = 0;
           break;
         case 9:    // C_f rows by the exact rule (mesh intersection)
-          launch(k_cf_rows_exact, nblk(P.nS, kCfWarps), 32 * kCfWarps, 0, s, P.nS, P.N, P.ntp, P.nt, P.tris, P.Xold,
-                 P.area, P.l2n, P.wall, P.cf_cap, P.cf_len, P.cf_col, P.cf_val, P.cf_val32, P.cflift, &P.ctl->aflags);
+          exact_rule_launch(P, s);
           *bytes = 0;
           break;
         case 10:   // fused finest-level launches, FP32: velocity down / up,
