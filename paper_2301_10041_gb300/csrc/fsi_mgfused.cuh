@@ -106,9 +106,9 @@ __host__ __device__ __forceinline__ int mf_tile_p(int N) { return N >= 512 ? 8 :
 // grids use 512 as well (1024 measured slower there).  Down frames have
 // TC + 8 plane entries a side (four planes), up frames TC + 4; a warp takes
 // two rows of up to 16 entries, four rows of up to 8.
-constexpr int mf_threads_ud(int tc) { return tc >= 16 ? 512 : (tc == 8 ? 512 : (tc == 4 ? 384 : 640)); }
-constexpr int mf_threads_uu(int tc) { return tc >= 16 ? 512 : (tc == 8 ? 512 : (tc == 4 ? 256 : 192)); }
-constexpr int mf_threads_p(int tp) { return tp >= 4 ? 256 : 128; }
+__host__ __device__ constexpr int mf_threads_ud(int tc) { return tc >= 8 ? 512 : 384; }
+__host__ __device__ constexpr int mf_threads_uu(int tc) { return tc >= 8 ? 512 : 256; }
+__host__ __device__ constexpr int mf_threads_p(int) { return 256; }   // either tile
 
 // Call f(integral_constant<degree>) for a Chebyshev degree 1 .. kMfMaxDeg
 // (the frame sizes and the step loops of the kernels are compile-time).
@@ -128,26 +128,22 @@ inline void mf_with_tile_u(int N, F&& f) {
   switch (mf_tile_u(N)) {
     case 16: f(std::integral_constant<int, 16>()); break;
     case 8: f(std::integral_constant<int, 8>()); break;
-    case 4: f(std::integral_constant<int, 4>()); break;
-    default: f(std::integral_constant<int, 2>()); break;
+    default: f(std::integral_constant<int, 4>()); break;
   }
 }
 template <class F>
 inline void mf_with_tile_p(int N, F&& f) {
-  switch (mf_tile_p(N)) {
-    case 8: f(std::integral_constant<int, 8>()); break;
-    case 4: f(std::integral_constant<int, 4>()); break;
-    case 2: f(std::integral_constant<int, 2>()); break;
-    default: f(std::integral_constant<int, 1>()); break;
-  }
+  if (mf_tile_p(N) == 8) f(std::integral_constant<int, 8>());
+  else f(std::integral_constant<int, 4>());
 }
 
-// Call f(integral_constant<CTAs per SM>) for a pressure launch (see the kernels).
+// Call f(integral_constant<tile>, integral_constant<CTAs per SM>) for a pressure
+// launch (see the kernels); only the pairs named here are compiled.
 template <bool UP, class F>
-inline void mf_with_minb_p(int N, F&& f) {
-  if (N <= 128) f(std::integral_constant<int, 1>());
-  else if (UP && N < 512) f(std::integral_constant<int, 8>());
-  else f(std::integral_constant<int, 6>());
+inline void mf_with_launch_p(int N, F&& f) {
+  if (N <= 128) f(std::integral_constant<int, 4>(), std::integral_constant<int, 1>());
+  else if (mf_tile_p(N) == 4) f(std::integral_constant<int, 4>(), std::integral_constant<int, UP ? 8 : 6>());
+  else f(std::integral_constant<int, 8>(), std::integral_constant<int, 6>());
 }
 
 template <class T>
@@ -366,7 +362,7 @@ __host__ __device__ __forceinline__ void mf_entries(int t, int ox, int oy, F&& f
     fn(r, e, ty, ox + 2 * px + (ty & 1), oy + 2 * py + (ty >> 1));
   }
 }
-constexpr int mf_rounds(int pw, int nt) { return (4 * pw * pw + nt - 1) / nt; }
+__host__ __device__ constexpr int mf_rounds(int pw, int nt) { return (4 * pw * pw + nt - 1) / nt; }
 
 // the value of vector v (node order) at the lattice node (ix, iy) of type t,
 // zero on the wall and outside

@@ -495,20 +495,22 @@ constexpr int kMfo64MinNFull = 64;   // full operator and Stokes residual
 // level says so, else the sliced-ELL kernel.
 template <class T>
 static void level_launch(const MGLevel<T>& L, int mode, const SpmvArgs<T>& a, cudaStream_t s) {
-  if (L.mfo.N > 0) {
-    const unsigned g = mfop_grid<T>(L.mfo.N);
-    if (mode == MODE_AXPBY) launch(k_mfv<T, MODE_AXPBY>, g, 128, 0, s, L.mfo, a);
-    else if (mode == MODE_CHEB) launch(k_mfv<T, MODE_CHEB>, g, 128, 0, s, L.mfo, a);
-    else if (mode == MODE_CHEB0) launch(k_mfv<T, MODE_CHEB0>, g, 128, 0, s, L.mfo, a);
-    else throw std::logic_error("level_launch");
-    return;
-  }
-  if (L.mfl) {
-    const unsigned g = nblk(3 * (size_t)L.N * L.N, 96);
-    if (mode == MODE_CHEB) launch(k_mfp<T, MODE_CHEB>, g, 96, 0, s, L.N, (const T*)L.mftab, a);
-    else if (mode == MODE_CHEB0) launch(k_mfp<T, MODE_CHEB0>, g, 96, 0, s, L.N, (const T*)L.mftab, a);
-    else throw std::logic_error("level_launch");
-    return;
+  if constexpr (std::is_same<T, double>::value) {   // the FP32 levels take the fused kernels
+    if (L.mfo.N > 0) {
+      const unsigned g = mfop_grid<T>(L.mfo.N);
+      if (mode == MODE_AXPBY) launch(k_mfv<T, MODE_AXPBY>, g, 128, 0, s, L.mfo, a);
+      else if (mode == MODE_CHEB) launch(k_mfv<T, MODE_CHEB>, g, 128, 0, s, L.mfo, a);
+      else if (mode == MODE_CHEB0) launch(k_mfv<T, MODE_CHEB0>, g, 128, 0, s, L.mfo, a);
+      else throw std::logic_error("level_launch");
+      return;
+    }
+    if (L.mfl) {
+      const unsigned g = nblk(3 * (size_t)L.N * L.N, 96);
+      if (mode == MODE_CHEB) launch(k_mfp<T, MODE_CHEB>, g, 96, 0, s, L.N, (const T*)L.mftab, a);
+      else if (mode == MODE_CHEB0) launch(k_mfp<T, MODE_CHEB0>, g, 96, 0, s, L.N, (const T*)L.mftab, a);
+      else throw std::logic_error("level_launch");
+      return;
+    }
   }
   sell_launch(L.A, mode, a, s);
 }
@@ -680,26 +682,27 @@ static void select_mf(MG<T>& mg, const HostSetup& hs, int mg_fused, bool count_o
                                     (int)mfu_up_smem<float>(TC, KD)));
           });
       };
-      auto pres = [](auto tp) {
+      auto pres_down = [](auto tp, auto mb) {
         for (int K = 1; K <= kMfMaxDeg; ++K)
           mf_with_degree(K, [&](auto kc) {
             constexpr int TP = decltype(tp)::value, KD = decltype(kc)::value, NT = mf_threads_p(TP);
-            for (int n : {128, 256, 512}) {
-              mf_with_minb_p<false>(n, [&](auto mb) {
-                CK(cudaFuncSetAttribute(k_mfp_down<float, TP, KD, NT, decltype(mb)::value>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)mfp_down_smem<float>(TP, KD)));
-              });
-              mf_with_minb_p<true>(n, [&](auto mb) {
-                CK(cudaFuncSetAttribute(k_mfp_up<float, TP, KD, NT, decltype(mb)::value>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)mfp_up_smem<float>(TP, KD)));
-              });
-            }
+            CK(cudaFuncSetAttribute(k_mfp_down<float, TP, KD, NT, decltype(mb)::value>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mfp_down_smem<float>(TP, KD)));
           });
       };
-      for (int N : {16, 64, 128, 512}) mf_with_tile_u(N, vel);   // every tile the maps choose
-      for (int N : {16, 64, 128, 512}) mf_with_tile_p(N, pres);
+      auto pres_up = [](auto tp, auto mb) {
+        for (int K = 1; K <= kMfMaxDeg; ++K)
+          mf_with_degree(K, [&](auto kc) {
+            constexpr int TP = decltype(tp)::value, KD = decltype(kc)::value, NT = mf_threads_p(TP);
+            CK(cudaFuncSetAttribute(k_mfp_up<float, TP, KD, NT, decltype(mb)::value>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mfp_up_smem<float>(TP, KD)));
+          });
+      };
+      for (int N : {32, 128, 256, 512}) {   // every kernel the maps choose
+        mf_with_tile_u(N, vel);
+        mf_with_launch_p<false>(N, pres_down);
+        mf_with_launch_p<true>(N, pres_up);
+      }
     });
   }
 }
@@ -723,8 +726,8 @@ static T* vcycle(MG<T>& mg, int l, cudaStream_t s, T* out, const SpmvArgs<T>* fi
 // residual and its restriction; the pre-smoothed iterate goes to L.x2, the
 // coarse right-hand side to C.b (and the coarse smoother start when the next
 // level runs the per-level sparse kernels).
-template <class T>
-static void mf_down_launch(MG<T>& mg, int l, const T* b, cudaStream_t s, const MfRes<T>* res = nullptr) {
+static void mf_down_launch(MG<float>& mg, int l, const float* b, cudaStream_t s, const MfRes<float>* res = nullptr) {
+  using T = float;
   const int last = (int)mg.lv.size() - 1;
   MGLevel<T>& L = mg.lv[l];
   MGLevel<T>& C = mg.lv[l + 1];
@@ -742,13 +745,12 @@ static void mf_down_launch(MG<T>& mg, int l, const T* b, cudaStream_t s, const M
     MfPresArgs<T> a;
     a.N = N; a.tab = L.mftab; a.ch = mf_cheb(L, K);
     a.b = b; a.xout = L.x2; a.bc = C.b; a.ci = ci; a.res = r;
-    mf_with_tile_p(N, [&](auto tp) {
+    mf_with_launch_p<false>(N, [&](auto tp, auto mb) {
       mf_with_degree(K, [&](auto kc) {
         constexpr int TP = decltype(tp)::value, KD = decltype(kc)::value, NT = mf_threads_p(TP);
         const unsigned g = nblk(N / 2, TP);
-        mf_with_minb_p<false>(N, [&](auto mb) {
-          launch(k_mfp_down<T, TP, KD, NT, decltype(mb)::value>, dim3(g, g), NT, mfp_down_smem<T>(TP, KD), s, a);
-        });
+        launch(k_mfp_down<T, TP, KD, NT, decltype(mb)::value>, dim3(g, g), NT,
+               mfp_down_smem<T>(TP, KD), s, a);
       });
     });
   } else {
@@ -767,8 +769,9 @@ static void mf_down_launch(MG<T>& mg, int l, const T* b, cudaStream_t s, const M
 
 // The up launch of fused level l: x = L.x2 + P xc, post-smoothing, result to
 // dst (never L.x2), with the epilogue fin.
-template <class T>
-static void mf_up_launch(MG<T>& mg, int l, const T* b, const T* xc, T* dst, const MfFin<T>* fin, cudaStream_t s) {
+static void mf_up_launch(MG<float>& mg, int l, const float* b, const float* xc, float* dst, const MfFin<float>* fin,
+                         cudaStream_t s) {
+  using T = float;
   MGLevel<T>& L = mg.lv[l];
   if (dst == L.x2) throw std::logic_error("mf_up_launch: the result may not overwrite the pre-smoothed iterate");
   const int N = L.N, K = mg.degree;
@@ -777,13 +780,12 @@ static void mf_up_launch(MG<T>& mg, int l, const T* b, const T* xc, T* dst, cons
     a.N = N; a.tab = L.mftab; a.ch = mf_cheb(L, K);
     a.b = b; a.xpre = L.x2; a.xc = xc; a.xout = dst;
     if (fin) a.fin = *fin;
-    mf_with_tile_p(N, [&](auto tp) {
+    mf_with_launch_p<true>(N, [&](auto tp, auto mb) {
       mf_with_degree(K, [&](auto kc) {
         constexpr int TP = decltype(tp)::value, KD = decltype(kc)::value, NT = mf_threads_p(TP);
         const unsigned g = nblk(N, 2 * TP);
-        mf_with_minb_p<true>(N, [&](auto mb) {
-          launch(k_mfp_up<T, TP, KD, NT, decltype(mb)::value>, dim3(g, g), NT, mfp_up_smem<T>(TP, KD), s, a);
-        });
+        launch(k_mfp_up<T, TP, KD, NT, decltype(mb)::value>, dim3(g, g), NT,
+               mfp_up_smem<T>(TP, KD), s, a);
       });
     });
   } else {
@@ -808,13 +810,17 @@ static void mf_up_launch(MG<T>& mg, int l, const T* b, const T* xc, T* dst, cons
 template <class T>
 static T* vcycle_mf(MG<T>& mg, int l, const T* b, cudaStream_t s, T* out, const MfFin<T>* fin,
                     const MfRes<T>* res = nullptr) {
-  MGLevel<T>& L = mg.lv[l];
-  MGLevel<T>& C = mg.lv[l + 1];
-  T* dst = out ? out : L.x;
-  mf_down_launch<T>(mg, l, b, s, res);
-  T* xc = C.mf ? vcycle_mf<T>(mg, l + 1, C.b, s, nullptr, nullptr) : vcycle<T>(mg, l + 1, s, (T*)nullptr);
-  mf_up_launch<T>(mg, l, res ? res->bout : b, xc, dst, fin, s);
-  return dst;
+  if constexpr (std::is_same<T, float>::value) {
+    MGLevel<T>& L = mg.lv[l];
+    MGLevel<T>& C = mg.lv[l + 1];
+    T* dst = out ? out : L.x;
+    mf_down_launch(mg, l, b, s, res);
+    T* xc = C.mf ? vcycle_mf<T>(mg, l + 1, C.b, s, nullptr, nullptr) : vcycle<T>(mg, l + 1, s, (T*)nullptr);
+    mf_up_launch(mg, l, res ? res->bout : b, xc, dst, fin, s);
+    return dst;
+  } else {
+    throw std::logic_error("the fused levels are FP32 (select_mf)");
+  }
 }
 
 // Algorithmic work of the fused launches of level l (not counting the work
@@ -1277,9 +1283,10 @@ static void stokes_velocity(Problem& P, Prec<T>& pr, const T* in_u, const T* p, 
     return;
   }
   if (zu) throw std::logic_error("stokes_velocity: the residual start needs the fused finest level");
-  if (p && L0u.mfo.N > 0) {
-    launch(k_mfv_start<T>, mfop_grid<T>(L0u.mfo.N), 128, 0, s, L0u.mfo, in_u, p, (const T*)L0u.dinv,
-           (T)L0u.ch.c0, L0u.b, L0u.d, L0u.x);
+  if (p && L0u.mfo.N > 0) {   // FP64 only, as in level_launch
+    if constexpr (std::is_same<T, double>::value)
+      launch(k_mfv_start<T>, mfop_grid<T>(L0u.mfo.N), 128, 0, s, L0u.mfo, in_u, p, (const T*)L0u.dinv,
+             (T)L0u.ch.c0, L0u.b, L0u.d, L0u.x);
   } else if (p) {
     SpmvArgs<T> a;
     a.x = p; a.y = L0u.b; a.z = in_u; a.alpha = -1; a.beta = 1;
@@ -3383,8 +3390,8 @@ int fsi_time_kernel(fsi_problem* h, int which, int reps, double* avg_ms, double*
           }
           MGLevel<float>& C = mg.lv[1];
           const bool up = (which & 1) != 0;
-          if (up) mf_up_launch<float>(mg, 0, L.b, C.x, L.x, nullptr, s);
-          else mf_down_launch<float>(mg, 0, L.b, s);
+          if (up) mf_up_launch(mg, 0, L.b, C.x, L.x, nullptr, s);
+          else mf_down_launch(mg, 0, L.b, s);
           *bytes = mf_work(P.hs, 0, which >= 12, up, mg.degree, sizeof(float)).bytes;
           break;
         }
