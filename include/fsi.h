@@ -134,8 +134,10 @@ typedef struct fsi_params {
                           at least 16 cells a side) each as two fused
                           launches (pre-smoothing + residual + restriction;
                           prolongation + post-smoothing), the FP64 levels of 32
-                          cells or more product by product; -1: the per-level
-                          sparse kernels on every level */
+                          cells or more product by product, the fluid rows of
+                          the operator in FP32 (from 4 cells) and in FP64
+                          (from 64); -1: the stored sparse matrices
+                          throughout */
     int    mg_coarse;  /* the coarsening stops at the first grid of at most
                           mg_coarse cells a side, whose operators are inverted
                           densely on the device when the problem is created

@@ -2291,7 +2291,9 @@ static void build_prec(Problem& P, Prec<T>& pr, const FullOp<T>& op, const doubl
   select_mf<T>(pr.mgU, P.hs, P.prm.mg_fused, ar.count_only);
   select_mf<T>(pr.mgP, P.hs, P.prm.mg_fused, ar.count_only);
   pr.op = op;
-  if (!f64 || P.N >= kMfo64MinNFull) pr.mf = make_mfop<T>(P.hs.levels[0]);
+  // mg_fused = -1 also keeps the stored fluid rows of the operator and of the
+  // Stokes residual: the assembled form that the matrix-free one is tested against
+  if (P.prm.mg_fused == 0 && (!f64 || P.N >= kMfo64MinNFull)) pr.mf = make_mfop<T>(P.hs.levels[0]);
   pr.Cs = upload_sell<T>(ar, to_sell(P.hs.Cs));
   pr.As = upload_sell<T>(ar, to_sell(P.hs.As));
   if (P.prm.solid_law == 1) {
