@@ -556,7 +556,9 @@ __global__ void __launch_bounds__(128) k_cf_apply(int nS, int cap, const int* __
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const T2 x = reinterpret_cast<const T2*>(a.x)[c[u]];
+      T2 x;
+      x.x = x.y = 0;
+      if (k0 + 4 * u < n) x = reinterpret_cast<const T2*>(a.x)[c[u]];   // 0 times an infinity would not be 0
       acc[0] += v[u] * x.x;
       acc[1] += v[u] * x.y;
     }

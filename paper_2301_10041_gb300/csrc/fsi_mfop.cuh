@@ -386,9 +386,11 @@ __global__ void __launch_bounds__(128) k_fullmv_mf(const __grid_constant__ FullO
         T2 l[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          const bool in = k + u < k1;
-          v[u] = in ? op.cft_val[k + u] : (T)0;
-          l[u] = lam[in ? op.cft_col[k + u] : 0];
+          v[u] = l[u].x = l[u].y = 0;
+          if (k + u < k1) {   // an absent entry reads nothing: 0 times an infinity would not be 0
+            v[u] = op.cft_val[k + u];
+            l[u] = lam[op.cft_col[k + u]];
+          }
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
