@@ -727,30 +727,28 @@ __global__ void __launch_bounds__(512) k_dense_sym(SymMap m, int ld, const T* __
   }
 }
 
-// the class matrices from the full inverse (rows of ldi entries); a row or
-// column whose representative lies on a mirror line and is odd there is zero
-template <class T>
-__global__ void k_sym_build(SymMap m, int ld, const double* __restrict__ G, int ldi, T* __restrict__ out) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y, cls = blockIdx.z;
-  if (q >= ld) return;
+// one class matrix (R rows of R entries) from the full inverse (rows of ldi
+// entries); a row or column whose representative lies on a mirror line and is odd
+// there is zero
+__global__ void k_sym_build(SymMap m, int cls, const double* __restrict__ G, int ldi, double* __restrict__ out) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
+  if (q >= m.R) return;
+  const int4 i = m.img[r], j = m.img[q];
+  const int sr = m.sgn[r], sq = m.sgn[q];
+  const double ca = (cls & 1) ? -1.0 : 1.0, cb = (cls & 2) ? -1.0 : 1.0;
+  const double ax = ca * ((sq & 1) ? -1.0 : 1.0), ay = cb * ((sq & 2) ? -1.0 : 1.0);
+  const bool zr = (i.y == i.x && ca * ((sr & 1) ? -1.0 : 1.0) < 0) || (i.z == i.x && cb * ((sr & 2) ? -1.0 : 1.0) < 0);
+  const bool zq = (j.y == j.x && ax < 0) || (j.z == j.x && ay < 0);
   double v = 0;
-  if (q < m.R) {
-    const int4 i = m.img[r], j = m.img[q];
-    const int sr = m.sgn[r], sq = m.sgn[q];
-    const double ca = (cls & 1) ? -1.0 : 1.0, cb = (cls & 2) ? -1.0 : 1.0;
-    const double ax = ca * ((sq & 1) ? -1.0 : 1.0), ay = cb * ((sq & 2) ? -1.0 : 1.0);
-    const bool zr = (i.y == i.x && ca * ((sr & 1) ? -1.0 : 1.0) < 0) || (i.z == i.x && cb * ((sr & 2) ? -1.0 : 1.0) < 0);
-    const bool zq = (j.y == j.x && ax < 0) || (j.z == j.x && ay < 0);
-    if (!zr && !zq) {
-      const double* g = G + (size_t)i.x * ldi;
-      v = g[j.x];
-      if (j.y != j.x) v += ax * g[j.y];
-      if (j.z != j.x) v += ay * g[j.z];
-      if (j.y != j.x && j.z != j.x) v += ax * ay * g[j.w];
-      v *= 0.25;
-    }
+  if (!zr && !zq) {
+    const double* g = G + (size_t)i.x * ldi;
+    v = g[j.x];
+    if (j.y != j.x) v += ax * g[j.y];
+    if (j.z != j.x) v += ay * g[j.z];
+    if (j.y != j.x && j.z != j.x) v += ax * ay * g[j.w];
+    v *= 0.25;
   }
-  out[((size_t)cls * m.R + r) * ld + q] = (T)v;
+  out[(size_t)r * m.R + q] = v;
 }
 
 // ------------------------------------------------ coarsest-level inverse

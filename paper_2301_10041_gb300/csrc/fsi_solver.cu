@@ -88,12 +88,17 @@ static void launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
 // ------------------------------------------------------------ device memory
 struct Arena {
   std::vector<void*> ptrs;
-  size_t bytes = 0;
+  size_t bytes = 0, peak = 0;   // held now, and at most so far
   bool count_only = false;
+  template <class T>
+  static size_t size(size_t n) {
+    return (std::max<size_t>(n, 1) * sizeof(T) + 255) & ~(size_t)255;
+  }
   template <class T>
   T* alloc(size_t n) {
     const size_t b = std::max<size_t>(n, 1) * sizeof(T);
-    bytes += (b + 255) & ~(size_t)255;
+    bytes += size<T>(n);
+    peak = std::max(peak, bytes);
     if (count_only) return nullptr;
     void* p = nullptr;
     if (cudaMalloc(&p, b) != cudaSuccess) throw std::bad_alloc();
@@ -105,6 +110,16 @@ struct Arena {
     T* d = alloc<T>(h.size());
     if (d && !h.empty()) CK(cudaMemcpy(d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice));
     return d;
+  }
+  // give back an array of n entries that only the creation of the problem needs
+  template <class T>
+  void drop(T*& p, size_t n) {
+    bytes -= size<T>(n);
+    if (p) {
+      ptrs.erase(std::find(ptrs.begin(), ptrs.end(), (void*)p));
+      CK(cudaFree(p));
+    }
+    p = nullptr;
   }
   void release() {
     for (void* p : ptrs) cudaFree(p);
@@ -334,7 +349,7 @@ struct ClusterMG {
 template <class T>
 struct MG {
   std::vector<MGLevel<T>> lv;
-  T* coarse_inv = nullptr;   // dense inverse of the coarsest level, rows of coarse_ld entries
+  T* coarse_inv = nullptr;   // dense inverse of the coarsest level, rows of coarse_ld entries (none with sym_inv)
   int coarse_n = 0;
   int coarse_ld = 0;         // coarse_n rounded up to 16 bytes (the row padding is zero)
   SymMap sym;                // its mirror images, and the class matrices (k_dense_sym)
@@ -353,17 +368,20 @@ constexpr double kChebRatioP = 8.0;
 // pivot (k_gj_step).  M holds the dense matrix on entry.
 static void dense_inverse_device(Arena& ar, double* M, int n, int ld, cudaStream_t s) {
   double* rc = ar.alloc<double>(4 * (size_t)n);   // row and column copies, two pairs
-  if (ar.count_only) return;
-  double *r0 = rc, *c0 = rc + n, *r1 = rc + 2 * n, *c1 = rc + 3 * n;
-  k_gj_first<<<nblk(n, 256), 256, 0, s>>>(n, ld, M, r0, c0);
-  CK(cudaGetLastError());
-  const dim3 blk(32, 8), grd((n + 31) / 32, (n + 7) / 8);
-  for (int k = 0; k < n; ++k) {
-    k_gj_step<<<grd, blk, 0, s>>>(n, ld, k, M, r0, c0, r1, c1);
-    std::swap(r0, r1);
-    std::swap(c0, c1);
+  if (!ar.count_only) {
+    double *r0 = rc, *c0 = rc + n, *r1 = rc + 2 * n, *c1 = rc + 3 * n;
+    k_gj_first<<<nblk(n, 256), 256, 0, s>>>(n, ld, M, r0, c0);
+    CK(cudaGetLastError());
+    const dim3 blk(32, 8), grd((n + 31) / 32, (n + 7) / 8);
+    for (int k = 0; k < n; ++k) {
+      k_gj_step<<<grd, blk, 0, s>>>(n, ld, k, M, r0, c0, r1, c1);
+      std::swap(r0, r1);
+      std::swap(c0, c1);
+    }
+    CK(cudaGetLastError());
+    CK(cudaStreamSynchronize(s));
   }
-  CK(cudaGetLastError());
+  ar.drop(rc, 4 * (size_t)n);
 }
 
 // 16-byte row length of the dense coarsest inverse, in entries
@@ -400,63 +418,96 @@ constexpr int kSymThreadsF32 = 256, kSymThreadsF64 = 512;   // two and four repr
 template <class T>
 constexpr int sym_threads() { return sizeof(T) == 8 ? kSymThreadsF64 : kSymThreadsF32; }
 
-// The coarsest level's dense inverse: the FP64 hierarchy inverts the
-// assembled matrix in place; the FP32 one rounds the FP64 inverse (inv64,
-// rows of ld64 entries).  The FP64 hierarchy is built first.
+// cluster-resident coarse levels, below
 template <class T>
-static void build_coarse_inverse(Arena& ar, const HostSetup& hs, bool pressure, MG<T>& mg, const double* inv64,
-                                 int ld64, cudaStream_t s) {
-  const int n = pressure ? hs.coarse_nL : hs.coarse_nA;
-  mg.coarse_n = n;
-  mg.coarse_ld = dense_ld<T>(n);
-  const int ld = mg.coarse_ld;
-  mg.coarse_inv = ar.alloc<T>((size_t)n * ld);
-  if constexpr (std::is_same<T, double>::value) {
-    if (!ar.count_only) {
-      const std::vector<double>& D = pressure ? hs.coarseL : hs.coarseA;
-      CK(cudaMemsetAsync(mg.coarse_inv, 0, (size_t)n * ld * sizeof(double), s));
-      CK(cudaMemcpy2DAsync(mg.coarse_inv, (size_t)ld * sizeof(double), D.data(), (size_t)n * sizeof(double),
-                           (size_t)n * sizeof(double), n, cudaMemcpyHostToDevice, s));
-    }
-    dense_inverse_device(ar, mg.coarse_inv, n, ld, s);
-  } else if (!ar.count_only) {
-    if (!inv64) throw std::logic_error("the FP64 coarse inverse is built first");
-    k_dense_round<T><<<dim3((ld + 255) / 256, n), 256, 0, s>>>(n, inv64, ld64, mg.coarse_inv, ld);
-    CK(cudaGetLastError());
-  }
-  // the class matrices of the dense product, from the FP64 inverse.  In FP32
-  // they pay from some 1500 unknowns on (1922: 2.93 -> 2.61 us, but 1058: 2.19 ->
-  // 2.38, 768: 1.69 -> 1.90, the class sums outweighing the shorter read); in FP64
-  // the multiply-adds saved always do (1922: 11.7 -> 7.3 us, 768: 5.6 -> 4.9).
-  if (sizeof(T) == 8 || n >= kSymMinF32) {
-    std::vector<int4> img;
-    std::vector<int> sgn;
-    sym_images(mg.lv.back().N, pressure, img, sgn);
-    mg.sym.R = (int)img.size();
-    mg.sym.img = ar.upload(img);
-    mg.sym.sgn = ar.upload(sgn);
-    mg.sym_ld = dense_ld<T>(mg.sym.R);
-    mg.sym_inv = ar.alloc<T>(4 * (size_t)mg.sym.R * mg.sym_ld);
-    if (!ar.count_only) {
-      const double* full = inv64;
-      int fld = ld64;
-      if constexpr (std::is_same<T, double>::value) {
-        full = mg.coarse_inv;
-        fld = ld;
-      }
-      k_sym_build<T><<<dim3(nblk(mg.sym_ld, 128), mg.sym.R, 4), 128, 0, s>>>(mg.sym, mg.sym_ld, full, fld, mg.sym_inv);
-      CK(cudaGetLastError());
-      if (4 * (size_t)mg.sym_ld * sizeof(T) > 48 * 1024)
-        CK(cudaFuncSetAttribute(k_dense_sym<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    }
-  }
-  // the coarsest right-hand side, padded to ld with zeros, for the dense product
-  MGLevel<T>& C = mg.lv.back();
-  C.b = ar.alloc<T>(ld);
+static void setup_cluster(Arena& ar, const HostSetup& hs, MG<T>& mg, bool pressure, int max_n);
+
+// The class matrices of the coarsest level, rounded from the FP64 ones (host,
+// 4 x R rows of R entries).
+template <class T>
+static void upload_classes(Arena& ar, MG<T>& mg, const SymMap& sym, const std::vector<double>& g) {
+  const int R = sym.R;
+  mg.sym = sym;
+  mg.sym_ld = dense_ld<T>(R);
+  const size_t ld = mg.sym_ld;
+  mg.sym_inv = ar.alloc<T>(4 * (size_t)R * ld);
+  if (ar.count_only) return;
+  std::vector<T> v(4 * (size_t)R * ld, (T)0);
+  for (size_t r = 0; r < 4 * (size_t)R; ++r)
+    for (int q = 0; q < R; ++q) v[r * ld + q] = (T)g[r * R + q];
+  CK(cudaMemcpy(mg.sym_inv, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice));
+  if (4 * ld * sizeof(T) > 48 * 1024)
+    CK(cudaFuncSetAttribute(k_dense_sym<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+}
+
+// The coarsest levels' solves of one hierarchy in both precisions (m32: null
+// without the FP32 one): the assembled matrix is inverted in place in FP64, and
+// what the V-cycles read is formed from that.  A hierarchy whose coarse levels
+// run as one cluster launch reads the full inverse; else the dense product takes
+// the class matrices (k_dense_sym) in FP64, and in FP32 from some 1500 unknowns on
+// (1922: 2.93 -> 2.61 us, but 1058: 2.19 -> 2.38, 768: 1.69 -> 1.90, the class sums
+// outweighing the shorter read; in FP64 the multiply-adds saved always pay, 1922:
+// 11.7 -> 7.3 us, 768: 5.6 -> 4.9).  The full FP64 inverse stays on the device only
+// where a cluster launch reads it, and the classes go through the host one at a time,
+// so that nothing but one class stands beside it: a mixed problem of 16 cells and
+// 271 solid nodes takes 32 MB at most, 73 with the inverses kept beside the classes.
+static void build_coarse(Arena& ar, const HostSetup& hs, bool pressure, MG<double>& m64, MG<float>* m32, int cl_max,
+                         cudaStream_t s) {
+  const int n = pressure ? hs.coarse_nL : hs.coarse_nA, ld = dense_ld<double>(n);
+  double* full = ar.alloc<double>((size_t)n * ld);
+  m64.coarse_n = n;
+  m64.coarse_ld = ld;
+  m64.coarse_inv = full;
   if (!ar.count_only) {
-    CK(cudaMemsetAsync(C.b, 0, (size_t)ld * sizeof(T), s));
+    const std::vector<double>& D = pressure ? hs.coarseL : hs.coarseA;
+    CK(cudaMemsetAsync(full, 0, (size_t)n * ld * sizeof(double), s));
+    CK(cudaMemcpy2DAsync(full, (size_t)ld * sizeof(double), D.data(), (size_t)n * sizeof(double),
+                         (size_t)n * sizeof(double), n, cudaMemcpyHostToDevice, s));
+  }
+  dense_inverse_device(ar, full, n, ld, s);
+  if (cl_max >= 0) setup_cluster<double>(ar, hs, m64, pressure, cl_max);
+  bool cls32 = false;
+  if (m32) {
+    m32->coarse_n = n;
+    m32->coarse_ld = dense_ld<float>(n);
+    if (cl_max >= 0) setup_cluster<float>(ar, hs, *m32, pressure, cl_max);
+    cls32 = !m32->cl.on && n >= kSymMinF32;
+    if (!cls32) {
+      m32->coarse_inv = ar.alloc<float>((size_t)n * m32->coarse_ld);
+      m32->cl.args.dense_inv = m32->coarse_inv;
+      if (!ar.count_only) {
+        k_dense_round<float><<<dim3((m32->coarse_ld + 255) / 256, n), 256, 0, s>>>(n, full, ld, m32->coarse_inv,
+                                                                                  m32->coarse_ld);
+        CK(cudaGetLastError());
+        CK(cudaStreamSynchronize(s));
+      }
+    }
+  }
+  const bool cls64 = !m64.cl.on;
+  if (!cls64 && !cls32) return;
+  SymMap sym;
+  std::vector<int4> img;
+  std::vector<int> sgn;
+  sym_images(hs.levels[(pressure ? hs.nlev_p : hs.nlev_u) - 1].N, pressure, img, sgn);
+  sym.R = (int)img.size();
+  sym.img = ar.upload(img);
+  sym.sgn = ar.upload(sgn);
+  const size_t RR = (size_t)sym.R * sym.R;
+  double* one = ar.alloc<double>(RR);
+  std::vector<double> g(ar.count_only ? 0 : 4 * RR);
+  for (int c = 0; c < 4 && !ar.count_only; ++c) {
+    k_sym_build<<<dim3(nblk(sym.R, 128), sym.R), 128, 0, s>>>(sym, c, full, ld, one);
+    CK(cudaGetLastError());
+    CK(cudaMemcpyAsync(g.data() + c * RR, one, RR * sizeof(double), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
   }
+  ar.drop(one, RR);
+  if (cls64) {
+    m64.coarse_inv = nullptr;
+    ar.drop(full, (size_t)n * ld);
+    upload_classes<double>(ar, m64, sym, g);
+  }
+  if (cls32) upload_classes<float>(ar, *m32, sym, g);
 }
 
 // The level's velocity stencils as MfOp; none (N = 0) when the grid has none or
@@ -515,9 +566,10 @@ static void level_launch(const MGLevel<T>& L, int mode, const SpmvArgs<T>& a, cu
   sell_launch(L.A, mode, a, s);
 }
 
+// What needs no device memory of a hierarchy: sizes, smoothing coefficients and
+// stencils of its levels.
 template <class T>
-static void build_mg(Arena& ar, const HostSetup& hs, bool pressure, int degree, MG<T>& mg, bool tune, bool mfree,
-                     cudaStream_t s, const double* inv64 = nullptr, int ld64 = 0) {
+static void plan_mg(const HostSetup& hs, bool pressure, int degree, MG<T>& mg, bool mfree) {
   const int nl = pressure ? hs.nlev_p : hs.nlev_u;
   mg.degree = degree;
   mg.pressure = pressure;
@@ -526,21 +578,8 @@ static void build_mg(Arena& ar, const HostSetup& hs, bool pressure, int degree, 
     const FluidLevelHost& H = hs.levels[l];
     MGLevel<T>& L = mg.lv[l];
     const HostBlockMatrix& A = pressure ? H.L : H.A;
-    const SellHost sa = to_sell(A);
-    L.A = upload_sell<T>(ar, sa);
-    if (tune && !ar.count_only) autotune_sell<T>(L.A, sa.soff[sa.nslices]);
     L.n = A.nrows * A.BR;
     L.N = H.N;
-    L.dinv = upload_as<T>(ar, pressure ? H.dinvL : H.dinvA);
-    if (l + 1 < nl) {
-      L.P = upload_sell<T>(ar, to_sell(pressure ? H.Pp : H.Pu));
-      L.R = upload_sell<T>(ar, to_sell(pressure ? H.Rp : H.Ru));
-      if (pressure) L.RA = upload_sell<T>(ar, to_sell(H.RAp));
-    }
-    L.x = ar.alloc<T>(L.n); L.x2 = ar.alloc<T>(L.n);
-    if (l + 1 < nl) L.b = ar.alloc<T>(L.n);   // the coarsest: build_coarse_inverse
-    if (!pressure) L.r = ar.alloc<T>(L.n);
-    L.d = ar.alloc<T>(L.n);
     const double hi = 1.05 * (pressure ? H.lmaxL : H.lmaxA);
     L.ch = cheb_coeffs(hi / (pressure ? kChebRatioP : kChebRatioU), hi, degree);
     if (H.mf)
@@ -561,6 +600,43 @@ static void build_mg(Arena& ar, const HostSetup& hs, bool pressure, int degree, 
         for (int c = 0; c < 2; ++c) L.mfu.dinv[t][c] = (T)H.dinvAt[t][c];
       }
     } else if (H.mf) {
+      L.mf_ok = true;
+      L.mfl = mfree && H.N >= kMfo64MinN;
+    }
+    if (mfree && !pressure && H.N >= kMfo64MinN) L.mfo = make_mfop<T>(H);
+  }
+}
+
+// Matrices and vectors of the levels, after build_coarse.
+template <class T>
+static void alloc_mg(Arena& ar, const HostSetup& hs, MG<T>& mg, bool tune, cudaStream_t s) {
+  const bool pressure = mg.pressure;
+  const int nl = (int)mg.lv.size();
+  for (int l = 0; l < nl; ++l) {
+    const FluidLevelHost& H = hs.levels[l];
+    MGLevel<T>& L = mg.lv[l];
+    const SellHost sa = to_sell(pressure ? H.L : H.A);
+    L.A = upload_sell<T>(ar, sa);
+    if (tune && !ar.count_only) autotune_sell<T>(L.A, sa.soff[sa.nslices]);
+    L.dinv = upload_as<T>(ar, pressure ? H.dinvL : H.dinvA);
+    if (l + 1 < nl) {
+      L.P = upload_sell<T>(ar, to_sell(pressure ? H.Pp : H.Pu));
+      L.R = upload_sell<T>(ar, to_sell(pressure ? H.Rp : H.Ru));
+      if (pressure) L.RA = upload_sell<T>(ar, to_sell(H.RAp));
+    }
+    L.x = ar.alloc<T>(L.n); L.x2 = ar.alloc<T>(L.n);
+    if (l + 1 < nl) {
+      L.b = ar.alloc<T>(L.n);
+    } else {   // the coarsest right-hand side, padded to the rows' length with zeros for the dense product
+      L.b = ar.alloc<T>(mg.coarse_ld);
+      if (!ar.count_only) {
+        CK(cudaMemsetAsync(L.b, 0, (size_t)mg.coarse_ld * sizeof(T), s));
+        CK(cudaStreamSynchronize(s));
+      }
+    }
+    if (!pressure) L.r = ar.alloc<T>(L.n);
+    L.d = ar.alloc<T>(L.n);
+    if (H.mf && pressure) {
       std::vector<double> tab(kMfPresTab);
       for (int v = 0; v < 9; ++v)
         for (int y = 0; y < 3; ++y)
@@ -569,12 +645,8 @@ static void build_mg(Arena& ar, const HostSetup& hs, bool pressure, int degree, 
       for (int v = 0; v < 9; ++v)
         for (int k = 0; k < 3; ++k) tab[kMfPresDinv + 3 * v + k] = H.dinvLv[v][k];
       L.mftab = upload_as<T>(ar, tab);
-      L.mf_ok = true;
-      L.mfl = mfree && H.N >= kMfo64MinN;
     }
-    if (mfree && !pressure && H.N >= kMfo64MinN) L.mfo = make_mfop<T>(H);
   }
-  build_coarse_inverse<T>(ar, hs, pressure, mg, inv64, ld64, s);
 }
 
 // ------------------------------------------- cluster-resident coarse levels
@@ -2266,30 +2338,36 @@ static fsi_params with_defaults(fsi_params p) {
   return p;
 }
 
-template <class T>
-static void build_prec(Problem& P, Prec<T>& pr, const FullOp<T>& op, const double* ref_xy) {
-  Arena& ar = P.ar;
-  const bool f64 = std::is_same<T, double>::value;
+// The four hierarchies' plans and coarsest solves, before any other memory is
+// taken: the full inverses that the creation needs go back before the rest comes.
+static void build_hierarchies(Problem& P) {
+  const bool mixed = P.prm.precision == 1;
   // the FP64 levels are matrix-free products launch by launch (the FP32 ones
   // take the fused kernels); mg_fused = -1 keeps the stored matrices
-  const bool mfree = f64 && P.prm.mg_fused == 0;
-  build_mg<T>(ar, P.hs, false, P.prm.mg_degree, pr.mgU, P.prm.autotune == 1, mfree, P.stream,
-              f64 ? nullptr : P.p64.mgU.coarse_inv, P.p64.mgU.coarse_ld);
-  build_mg<T>(ar, P.hs, true, P.prm.mg_degree, pr.mgP, P.prm.autotune == 1, mfree, P.stream,
-              f64 ? nullptr : P.p64.mgP.coarse_inv, P.p64.mgP.coarse_ld);
+  const bool mfree = P.prm.mg_fused == 0;
   // With the matrix-free levels the automatic choice leaves the cluster out:
   // two fused launches per level measured faster than the cluster launch of
   // the same levels in FP32 (10.8 against 9.7 steps/s on the 128 x 128
   // cavity), and in FP64 the pressure cluster from 32 cells down takes 42 us
   // where its levels launch by launch take 20.
   int cl_max = P.prm.mg_cluster;
-  if (cl_max == 0 && P.prm.mg_fused == 0) cl_max = 8;
-  if (cl_max >= 0) {
-    setup_cluster<T>(ar, P.hs, pr.mgU, false, cl_max);
-    setup_cluster<T>(ar, P.hs, pr.mgP, true, cl_max);
+  if (cl_max == 0 && mfree) cl_max = 8;
+  for (bool pressure : {false, true}) {
+    MG<double>& m64 = pressure ? P.p64.mgP : P.p64.mgU;
+    MG<float>& m32 = pressure ? P.p32.mgP : P.p32.mgU;
+    plan_mg<double>(P.hs, pressure, P.prm.mg_degree, m64, mfree);
+    if (mixed) plan_mg<float>(P.hs, pressure, P.prm.mg_degree, m32, false);
+    build_coarse(P.ar, P.hs, pressure, m64, mixed ? &m32 : nullptr, cl_max, P.stream);
+    if (mixed) select_mf<float>(m32, P.hs, P.prm.mg_fused, P.ar.count_only);
   }
-  select_mf<T>(pr.mgU, P.hs, P.prm.mg_fused, ar.count_only);
-  select_mf<T>(pr.mgP, P.hs, P.prm.mg_fused, ar.count_only);
+}
+
+template <class T>
+static void build_prec(Problem& P, Prec<T>& pr, const FullOp<T>& op, const double* ref_xy) {
+  Arena& ar = P.ar;
+  const bool f64 = std::is_same<T, double>::value;
+  alloc_mg<T>(ar, P.hs, pr.mgU, P.prm.autotune == 1, P.stream);
+  alloc_mg<T>(ar, P.hs, pr.mgP, P.prm.autotune == 1, P.stream);
   pr.op = op;
   // mg_fused = -1 also keeps the stored fluid rows of the operator and of the
   // Stokes residual: the assembled form that the matrix-free one is tested against
@@ -2604,6 +2682,7 @@ static void allocate_problem(Problem& P, const double* ref_xy, const int* tris_h
   Arena& ar = P.ar;
   const HostSetup& hs = P.hs;
   const int npe = elem_nodes(P.prm);
+  build_hierarchies(P);
   P.tris = ar.upload(std::vector<int>(tris_h, tris_h + npe * (size_t)P.nTri));
   P.area = ar.upload(npe == 4 ? hs.pt_w : hs.tri_area);
   P.ntp = ar.upload(hs.node_tri_ptr);
@@ -2783,7 +2862,7 @@ static size_t footprint_impl(const fsi_params& prm0, int n_nodes, int n_tris, co
   sp.coarse_max_p = prm.mg_coarse_p;
   build_setup(sp, n_nodes, n_tris, ref_xy, tris, P.hs);
   allocate_problem(P, ref_xy, tris);
-  return P.ar.bytes;
+  return P.ar.peak;
 }
 
 extern "C" {
