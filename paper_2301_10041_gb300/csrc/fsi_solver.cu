@@ -607,7 +607,13 @@ static void plan_mg(const HostSetup& hs, bool pressure, int degree, MG<T>& mg, b
   }
 }
 
-// Matrices and vectors of the levels, after build_coarse.
+// Vectors of the levels and the matrices that the V-cycle reads, after
+// build_coarse and select_mf: none on the coarsest level (dense product), on the
+// fused levels and in the cluster (their own images; a count without a device takes
+// the cluster for granted and so counts its levels here too), and not A where the
+// level's product is matrix-free.  With the level-0 rows of the operator, which
+// make_op leaves out likewise: 7.5 -> 4.4 GB on 512 cells in mixed precision with
+// 60 basis vectors.
 template <class T>
 static void alloc_mg(Arena& ar, const HostSetup& hs, MG<T>& mg, bool tune, cudaStream_t s) {
   const bool pressure = mg.pressure;
@@ -615,11 +621,14 @@ static void alloc_mg(Arena& ar, const HostSetup& hs, MG<T>& mg, bool tune, cudaS
   for (int l = 0; l < nl; ++l) {
     const FluidLevelHost& H = hs.levels[l];
     MGLevel<T>& L = mg.lv[l];
-    const SellHost sa = to_sell(pressure ? H.L : H.A);
-    L.A = upload_sell<T>(ar, sa);
-    if (tune && !ar.count_only) autotune_sell<T>(L.A, sa.soff[sa.nslices]);
+    const bool stored = l + 1 < nl && !L.mf && !(mg.cl.on && l >= mg.cl.lc && !ar.count_only);
+    if (stored && !L.mfl && L.mfo.N == 0) {
+      const SellHost sa = to_sell(pressure ? H.L : H.A);
+      L.A = upload_sell<T>(ar, sa);
+      if (tune && !ar.count_only) autotune_sell<T>(L.A, sa.soff[sa.nslices]);
+    }
     L.dinv = upload_as<T>(ar, pressure ? H.dinvL : H.dinvA);
-    if (l + 1 < nl) {
+    if (stored) {
       L.P = upload_sell<T>(ar, to_sell(pressure ? H.Pp : H.Pu));
       L.R = upload_sell<T>(ar, to_sell(pressure ? H.Rp : H.Ru));
       if (pressure) L.RA = upload_sell<T>(ar, to_sell(H.RAp));
@@ -634,7 +643,7 @@ static void alloc_mg(Arena& ar, const HostSetup& hs, MG<T>& mg, bool tune, cudaS
         CK(cudaStreamSynchronize(s));
       }
     }
-    if (!pressure) L.r = ar.alloc<T>(L.n);
+    if (stored && !pressure) L.r = ar.alloc<T>(L.n);
     L.d = ar.alloc<T>(L.n);
     if (H.mf && pressure) {
       std::vector<double> tab(kMfPresTab);
@@ -2360,18 +2369,18 @@ static void build_hierarchies(Problem& P) {
     build_coarse(P.ar, P.hs, pressure, m64, mixed ? &m32 : nullptr, cl_max, P.stream);
     if (mixed) select_mf<float>(m32, P.hs, P.prm.mg_fused, P.ar.count_only);
   }
+  // mg_fused = -1 also keeps the stored fluid rows of the operator and of the
+  // Stokes residual: the assembled form that the matrix-free one is tested against
+  if (mfree && P.N >= kMfo64MinNFull) P.p64.mf = make_mfop<double>(P.hs.levels[0]);
+  if (mfree && mixed) P.p32.mf = make_mfop<float>(P.hs.levels[0]);
 }
 
 template <class T>
 static void build_prec(Problem& P, Prec<T>& pr, const FullOp<T>& op, const double* ref_xy) {
   Arena& ar = P.ar;
-  const bool f64 = std::is_same<T, double>::value;
   alloc_mg<T>(ar, P.hs, pr.mgU, P.prm.autotune == 1, P.stream);
   alloc_mg<T>(ar, P.hs, pr.mgP, P.prm.autotune == 1, P.stream);
   pr.op = op;
-  // mg_fused = -1 also keeps the stored fluid rows of the operator and of the
-  // Stokes residual: the assembled form that the matrix-free one is tested against
-  if (P.prm.mg_fused == 0 && (!f64 || P.N >= kMfo64MinNFull)) pr.mf = make_mfop<T>(P.hs.levels[0]);
   pr.Cs = upload_sell<T>(ar, to_sell(P.hs.Cs));
   pr.As = upload_sell<T>(ar, to_sell(P.hs.As));
   if (P.prm.solid_law == 1) {
@@ -2397,15 +2406,21 @@ static void build_prec(Problem& P, Prec<T>& pr, const FullOp<T>& op, const doubl
   pr.stokes_omega = (T)P.prm.stokes_omega;
 }
 
+// The operator's structure; the stored fluid rows only where they are read
+// (pr.mf: not by the products; -B^T also starts the velocity V-cycle of a finest
+// level that is neither fused nor matrix-free).
 template <class T>
-static FullOp<T> make_op(Problem& P, const T* cfv, const T* cftv) {
+static FullOp<T> make_op(Problem& P, const Prec<T>& pr, const T* cfv, const T* cftv) {
   Arena& ar = P.ar;
   FullOp<T> op;
   op.nU = P.nU; op.nP = P.nP; op.nS = P.nS;
   op.gU = nblk(P.nU, 32); op.gP = nblk(P.nP, 32); op.gS = nblk(P.nS, 32);
-  op.Af = upload_sell<T>(ar, to_sell(P.hs.levels[0].A));
-  op.Bt = upload_sell<T>(ar, to_sell(P.hs.Bt));
-  op.Bneg = upload_sell<T>(ar, to_sell(P.hs.Bneg));
+  const MGLevel<T>& L0 = pr.mgU.lv[0];
+  if (pr.mf.N == 0) {
+    op.Af = upload_sell<T>(ar, to_sell(P.hs.levels[0].A));
+    op.Bneg = upload_sell<T>(ar, to_sell(P.hs.Bneg));
+  }
+  if (pr.mf.N == 0 || !(L0.mf || L0.mfo.N > 0)) op.Bt = upload_sell<T>(ar, to_sell(P.hs.Bt));
   op.Ssol = upload_sell<T>(ar, to_sell(P.hs.Ssol));
   op.cft_ptr = P.cft_ptr; op.cft_col = P.cft_col; op.cft_val = cftv;
   op.cf_len = P.cf_len; op.cf_col = P.cf_col; op.cf_val = cfv; op.cf_cap = P.cf_cap;
@@ -2769,10 +2784,10 @@ static void allocate_problem(Problem& P, const double* ref_xy, const int* tris_h
   P.red_blocks = red_grid(P.n);
   P.part = ar.alloc<double>((size_t)std::max(P.red_blocks, 64) * (m + 2));
   P.ctl = ar.alloc<Ctl>(1);
-  P.op64 = make_op<double>(P, P.cf_val, P.cft_val);
+  P.op64 = make_op<double>(P, P.p64, P.cf_val, P.cft_val);
   build_prec<double>(P, P.p64, P.op64, ref_xy);
   if (P.prm.precision == 1) {
-    P.op32 = make_op<float>(P, P.cf_val32, P.cft_val32);
+    P.op32 = make_op<float>(P, P.p32, P.cf_val32, P.cft_val32);
     build_prec<float>(P, P.p32, P.op32, ref_xy);
   }
 }
@@ -3416,6 +3431,21 @@ int fsi_time_kernel(fsi_problem* h, int which, int reps, double* avg_ms, double*
     double total = 0;
     cudaStream_t s = P.stream;
     const HostBlockMatrix& A0 = P.hs.levels[0].A;
+    // the stored matrix of the smoothing steps, for the timing alone
+    struct Held : Arena {
+      ~Held() { release(); }
+    } held;
+    Sell<float> A2;
+    Sell<double> A3;
+    if (which == 2 || which == 3) {
+      const SellHost sa = to_sell(A0);
+      if (which == 2) A2 = upload_sell<float>(held, sa);
+      else A3 = upload_sell<double>(held, sa);
+      if (P.prm.autotune == 1) {
+        if (which == 2) autotune_sell<float>(A2, sa.soff[sa.nslices]);
+        else autotune_sell<double>(A3, sa.soff[sa.nslices]);
+      }
+    }
     for (int r = 0; r < reps + 1; ++r) {
       if (which < 4 || which >= 10) launch(k_flush, 2 * 152, 512, 0, s, flush_n, fl, (unsigned)r);
       CK(cudaEventRecord(e0, s));
@@ -3428,19 +3458,19 @@ int fsi_time_kernel(fsi_problem* h, int which, int reps, double* avg_ms, double*
           full_launch<double, double>(P.p64, P.x, P.w, P.b, -1.0, 1.0, nullptr, 0, nullptr, s);
           *bytes = fullop_bytes<double>(P, P.p64.mf.N > 0, cfnnz, 16, 8);
           break;
-        case 2: {  // finest velocity Chebyshev step, FP32
+        case 2: {  // finest velocity Chebyshev step on the stored matrix, FP32
           MGLevel<float>& L = P.p32.mgU.lv[0];
           SpmvArgs<float> a;
           a.x = L.x; a.y = L.x2; a.z = L.b; a.d = L.d; a.dinv = L.dinv; a.c1 = 0.5f; a.c2 = 0.5f;
-          sell_launch(L.A, MODE_CHEB, a, s);
+          sell_launch(A2, MODE_CHEB, a, s);
           *bytes = sell_bytes<float>(A0) + 6.0 * L.n * sizeof(float);
           break;
         }
-        case 3: {  // finest velocity Chebyshev step, FP64
+        case 3: {  // the same, FP64
           MGLevel<double>& L = P.p64.mgU.lv[0];
           SpmvArgs<double> a;
           a.x = L.x; a.y = L.x2; a.z = L.b; a.d = L.d; a.dinv = L.dinv; a.c1 = 0.5; a.c2 = 0.5;
-          sell_launch(L.A, MODE_CHEB, a, s);
+          sell_launch(A3, MODE_CHEB, a, s);
           *bytes = sell_bytes<double>(A0) + 6.0 * L.n * sizeof(double);
           break;
         }

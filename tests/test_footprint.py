@@ -55,3 +55,17 @@ def test_budgets_of_the_stored_form_still_admit(N, rings, opt, counts, mesh):
     assert _admits(fsi, prm, xy, tris, mesh)
     assert _admits(fsi, prm, xy, tris, by_counts)       # the counts bound every mesh
     assert not _admits(fsi, prm, xy, tris, by_counts // 4)
+
+
+@pytest.mark.parametrize("N,rings,opt,counts", [
+    (128, 25, dict(precision=1, restart=60), 516639744),
+    (128, 25, dict(precision=0, restart=60), 458216960),
+])
+def test_matrix_free_levels_hold_no_stored_matrices(N, rings, opt, counts):
+    """Neither the operator nor the finest level keeps its velocity block (2 x 2
+    values and a column per block, 16 blocks a row: one of each at least)."""
+    fsi = _library()
+    xy, tris = fi.ring_disk_mesh(rings, 0.2, (0.47, 0.52))
+    by_counts = fsi.footprint_bytes(_params(fsi, N, opt), xy.shape[0], tris.shape[0])
+    block = 4 * (4 if opt["precision"] else 8) + 4
+    assert counts - by_counts >= 2 * 15 * (2 * N - 1) ** 2 * block
