@@ -369,8 +369,9 @@ __device__ __forceinline__ void exact_load(const int* __restrict__ tris, const d
   }
 }
 
-// The pairs of every triangle that overlaps at most kExactCells cells (a body
-// refined with the fluid grid has no other), for its three vertices at once: the
+// The pairs of every triangle that overlaps at most kExactCells cells (of a body
+// refined with the fluid grid all but a few: 0.05 % of the triangles overlap more on
+// the 128-cell cavity), for its three vertices at once: the
 // clip, the points and the basis of a pair serve three rows, which took them
 // three times over when each row formed its own.  Bound by the FP64 pipe, as the
 // rows were: assembly on 256 cells (63 654 triangles) 2.69 -> 1.23 ms, 0.27 ms on
@@ -405,7 +406,7 @@ __global__ void __launch_bounds__(128) k_exact_pairs(int n_tris, int N, const in
 // S4 with the paper's exact rule (Section 4): one warp per solid node l.
 // Every (triangle of l, fluid cell of the triangle's bounding box) pair is one
 // work item (read from k_exact_pairs, or formed here for a triangle over more than
-// kExactCells cells); the lanes take 32 items at a time, and their 9 contributions are
+// kExactCells cells, and without the table); the lanes take 32 items at a time, and their 9 contributions are
 // added to the row window in item order (no atomics, deterministic), then
 // compacted as in k_cf_rows.  A vertex outside [0,1]^2 raises
 // FLAG_OUT_OF_DOMAIN; more than 32 triangles at a node or a window above
@@ -481,7 +482,7 @@ __global__ void __launch_bounds__(32 * kCfWarps) k_cf_rows_exact(
       const int bx0 = __shfl_sync(0xffffffffu, cx0, k), by0 = __shfl_sync(0xffffffffu, cy0, k);
       const int bwk = __shfl_sync(0xffffffffu, bw, k), ek = __shfl_sync(0xffffffffu, excl, k);
       const int ck = __shfl_sync(0xffffffffu, cnt, k);
-      if (i < nitems && ck <= kExactCells) {
+      if (i < nitems && pairs && ck <= kExactCells) {
         const int j = i - ek;
         cx = bx0 + j % bwk;
         cy = by0 + j / bwk;

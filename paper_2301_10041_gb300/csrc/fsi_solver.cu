@@ -89,6 +89,10 @@ static void launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
 struct Arena {
   std::vector<void*> ptrs;
   size_t bytes = 0, peak = 0;   // held now, and at most so far
+  // bytes less than the form with every matrix and the full coarsest inverses
+  // stored takes: what the tables that replace work by memory may take, so that a
+  // budget for that form still admits the problem
+  long long spared = 0;
   bool count_only = false;
   template <class T>
   static size_t size(size_t n) {
@@ -167,6 +171,12 @@ template <class T>
 static T* upload_as(Arena& ar, const std::vector<double>& h) {
   std::vector<T> v(h.begin(), h.end());
   return ar.upload(v);
+}
+
+// values and columns of a matrix's stored blocks: what leaving it out spares at least
+template <class T>
+static double sell_bytes(const HostBlockMatrix& A) {
+  return (double)A.nnzb() * (A.NV * sizeof(T) + sizeof(int));
 }
 
 // ------------------------------------------------------------- SpMV launch
@@ -431,6 +441,7 @@ static void upload_classes(Arena& ar, MG<T>& mg, const SymMap& sym, const std::v
   mg.sym_ld = dense_ld<T>(R);
   const size_t ld = mg.sym_ld;
   mg.sym_inv = ar.alloc<T>(4 * (size_t)R * ld);
+  ar.spared -= Arena::size<T>(4 * (size_t)R * ld);
   if (ar.count_only) return;
   std::vector<T> v(4 * (size_t)R * ld, (T)0);
   for (size_t r = 0; r < 4 * (size_t)R; ++r)
@@ -492,6 +503,7 @@ static void build_coarse(Arena& ar, const HostSetup& hs, bool pressure, MG<doubl
   sym.R = (int)img.size();
   sym.img = ar.upload(img);
   sym.sgn = ar.upload(sgn);
+  ar.spared -= Arena::size<int4>(img.size()) + Arena::size<int>(sgn.size());
   const size_t RR = (size_t)sym.R * sym.R;
   double* one = ar.alloc<double>(RR);
   std::vector<double> g(ar.count_only ? 0 : 4 * RR);
@@ -505,9 +517,13 @@ static void build_coarse(Arena& ar, const HostSetup& hs, bool pressure, MG<doubl
   if (cls64) {
     m64.coarse_inv = nullptr;
     ar.drop(full, (size_t)n * ld);
+    ar.spared += Arena::size<double>((size_t)n * ld);
     upload_classes<double>(ar, m64, sym, g);
   }
-  if (cls32) upload_classes<float>(ar, *m32, sym, g);
+  if (cls32) {
+    ar.spared += Arena::size<float>((size_t)n * m32->coarse_ld);
+    upload_classes<float>(ar, *m32, sym, g);
+  }
 }
 
 // The level's velocity stencils as MfOp; none (N = 0) when the grid has none or
@@ -626,6 +642,8 @@ static void alloc_mg(Arena& ar, const HostSetup& hs, MG<T>& mg, bool tune, cudaS
       const SellHost sa = to_sell(pressure ? H.L : H.A);
       L.A = upload_sell<T>(ar, sa);
       if (tune && !ar.count_only) autotune_sell<T>(L.A, sa.soff[sa.nslices]);
+    } else if (!(mg.cl.on && l >= mg.cl.lc)) {
+      ar.spared += (long long)sell_bytes<T>(pressure ? H.L : H.A);
     }
     L.dinv = upload_as<T>(ar, pressure ? H.dinvL : H.dinvA);
     if (stored) {
@@ -1100,7 +1118,7 @@ struct Problem {
   int* l2n = nullptr; double* wall = nullptr;
   int* cell = nullptr; double* xi = nullptr; double* eta = nullptr;
   int cf_cap = 64;
-  double* pairs = nullptr;   // exact rule: contributions per (triangle, cell) pair (k_exact_pairs)
+  double* pairs = nullptr;   // exact rule: contributions per (triangle, cell) pair (k_exact_pairs), or none
   // nonlinear solid: reference gradients of the P1 basis per triangle (3 x 2),
   // tangent blocks in the slots of the solid pair matrix (4 per slot)
   double* tgrad = nullptr;
@@ -2419,6 +2437,8 @@ static FullOp<T> make_op(Problem& P, const Prec<T>& pr, const T* cfv, const T* c
   if (pr.mf.N == 0) {
     op.Af = upload_sell<T>(ar, to_sell(P.hs.levels[0].A));
     op.Bneg = upload_sell<T>(ar, to_sell(P.hs.Bneg));
+  } else {
+    ar.spared += (long long)(sell_bytes<T>(P.hs.levels[0].A) + sell_bytes<T>(P.hs.Bneg));
   }
   if (pr.mf.N == 0 || !(L0.mf || L0.mfo.N > 0)) op.Bt = upload_sell<T>(ar, to_sell(P.hs.Bt));
   op.Ssol = upload_sell<T>(ar, to_sell(P.hs.Ssol));
@@ -2448,9 +2468,11 @@ static KrylovArgs krylov_args(Problem& P, cudaGraphConditionalHandle h) {
   return k;
 }
 
-// S4 by the exact rule: the pairs of small triangles, then the C_f rows.
+// S4 by the exact rule: the pairs of small triangles (when there is room for them),
+// then the C_f rows.
 static void exact_rule_launch(Problem& P, cudaStream_t s) {
-  launch(k_exact_pairs, nblk((size_t)kExactCells * P.nTri, 128), 128, 0, s, P.nTri, P.N, P.tris, P.Xold, P.area, P.pairs);
+  if (P.pairs)
+    launch(k_exact_pairs, nblk((size_t)kExactCells * P.nTri, 128), 128, 0, s, P.nTri, P.N, P.tris, P.Xold, P.area, P.pairs);
   launch(k_cf_rows_exact, nblk(P.nS, kCfWarps), 32 * kCfWarps, 0, s, P.nS, P.N, P.ntp, P.nt, P.tris, P.Xold, P.area,
          P.l2n, P.wall, P.cf_cap, P.cf_len, P.cf_col, P.cf_val, P.cf_val32, P.cflift, &P.ctl->aflags, P.pairs, P.nTri);
 }
@@ -2704,7 +2726,6 @@ static void allocate_problem(Problem& P, const double* ref_xy, const int* tris_h
   P.nt = ar.upload(hs.node_tri);
   P.l2n = ar.upload(hs.lattice_to_node);
   P.wall = ar.upload(hs.wall_u);
-  if (P.prm.coupling == 1) P.pairs = ar.alloc<double>(27 * (size_t)kExactCells * P.nTri);
   P.cell = ar.alloc<int>(P.nPts);
   P.xi = ar.alloc<double>(P.nPts);
   P.eta = ar.alloc<double>(P.nPts);
@@ -2790,15 +2811,22 @@ static void allocate_problem(Problem& P, const double* ref_xy, const int* tris_h
     P.op32 = make_op<float>(P, P.p32, P.cf_val32, P.cft_val32);
     build_prec<float>(P, P.p32, P.op32, ref_xy);
   }
+  // The pairs of the exact rule live in the Krylov basis, idle while C_f is
+  // assembled; where it is too short (few vectors, a body much finer than the grid)
+  // they take memory spared elsewhere, or each row forms its own.
+  if (P.prm.coupling == 1) {
+    const size_t np = 27 * (size_t)kExactCells * P.nTri;
+    if ((size_t)(P.m + 1) * P.n >= np) {
+      P.pairs = P.V;
+    } else if ((long long)Arena::size<double>(np) <= ar.spared) {
+      ar.spared -= Arena::size<double>(np);
+      P.pairs = ar.alloc<double>(np);
+    }
+  }
 }
 
 
 // ----------------------------------------------------------- timing hook
-template <class T>
-static double sell_bytes(const HostBlockMatrix& A) {
-  return (double)A.nnzb() * (A.NV * sizeof(T) + sizeof(int));  // stored blocks: values + column index
-}
-
 template <class T>
 static double fullop_bytes(Problem& P, bool mf, double cfnnz, size_t xbytes, size_t ybytes) {
   const HostSetup& hs = P.hs;

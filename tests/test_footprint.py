@@ -19,6 +19,10 @@ COARSE = [   # the coarsest inverses
     (64, 9, dict(precision=1, restart=60), 157438720, 150683684),
     (64, 9, dict(precision=0, restart=60, mg_coarse=32), 673263104, 666547493),
 ]
+PAIRS = [    # the exact rule's table of pairs
+    (128, 50, dict(precision=1, restart=60, mg_fused=-1, coupling=1), 735133952, None),
+    (16, 30, dict(precision=1, restart=60, coupling=1), 76600320, 73876072),
+]
 
 
 def _library():
@@ -45,14 +49,14 @@ def _admits(fsi, prm, xy, tris, budget):
         return e.code != fsi.FSI_ERR_BUDGET
 
 
-@pytest.mark.parametrize("N,rings,opt,counts,mesh", COARSE)
+@pytest.mark.parametrize("N,rings,opt,counts,mesh", COARSE + PAIRS)
 def test_budgets_of_the_stored_form_still_admit(N, rings, opt, counts, mesh):
     fsi = _library()
     xy, tris = fi.ring_disk_mesh(rings, 0.2, (0.47, 0.52))
     prm = _params(fsi, N, opt)
     by_counts = fsi.footprint_bytes(prm, xy.shape[0], tris.shape[0])
     assert 0 < by_counts <= counts
-    assert _admits(fsi, prm, xy, tris, mesh)
+    assert mesh is None or _admits(fsi, prm, xy, tris, mesh)
     assert _admits(fsi, prm, xy, tris, by_counts)       # the counts bound every mesh
     assert not _admits(fsi, prm, xy, tris, by_counts // 4)
 
