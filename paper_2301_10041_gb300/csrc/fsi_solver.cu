@@ -1106,6 +1106,7 @@ struct Problem {
   cudaStream_t stream = nullptr, s2 = nullptr, s3 = nullptr, s4 = nullptr, s5 = nullptr;  // capture helpers
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_fork2 = nullptr, ev_join2 = nullptr;
   bool own_stream = false;
+  bool by_counts = false;   // a footprint count without the mesh itself
   int device = 0;
   Arena ar;
   HostSetup hs;
@@ -1201,22 +1202,36 @@ static void solid_patch_solve(Prec<T>& pr, const T* bsrc, T scale, const Sell<T>
 }
 
 // The patches of a problem's body on the device; none (np = 0) when the mesh
-// does not suit.  A footprint count without the mesh itself takes a bound.
+// does not suit or they take more than the counts' bound (planar growth of the
+// planned patches, with room for rows of kScWide entries) or than the memory spared
+// elsewhere (a body much finer than the grid).  A footprint by counts alone (no
+// mesh) takes that most of them.
 template <class T>
-static void setup_solid_patches(Arena& ar, const HostSetup& hs, const double* ref_xy, Prec<T>& pr) {
+static void setup_solid_patches(Arena& ar, const HostSetup& hs, const double* ref_xy, bool by_counts, Prec<T>& pr) {
   constexpr bool f64 = std::is_same<T, double>::value;
   constexpr int NT = sc_threads<T>();
-  SolidPatchHost h;
-  if (!build_solid_patches(hs.Cs, ref_xy, pr.cs_k - 1, f64, NT, h) ||
-      4 * sizeof(T) * (size_t)h.max_loc > kClSmemCap) {   // an outer layer too long for the iterate's two copies
-    if (ar.count_only) {
-      const SolidPlan pl = plan_solid_patches(hs.Cs.nrows, pr.cs_k - 1, f64, 2 * NT);
-      const double r = std::sqrt((double)hs.Cs.nrows / std::max(1, pl.np)) + 2.0 * pl.steps;
-      const double loc = pl.np * std::min((double)hs.Cs.nrows, r * r);
-      ar.bytes += (size_t)(1.3 * loc * (kScWide * (sizeof(T) + 2) + 4)) + 4096;
-    }
+  const SolidPlan pl = plan_solid_patches(hs.Cs.nrows, pr.cs_k - 1, f64, 2 * NT);
+  if (pl.np == 0) return;
+  const double r = std::sqrt((double)hs.Cs.nrows / pl.np) + 2.0 * pl.steps;
+  const double loc = pl.np * std::min((double)hs.Cs.nrows, r * r);
+  const long long bound = (long long)(1.3 * loc * (kScWide * (sizeof(T) + 2) + 4)) + 4096 +
+                          (pl.launches > 1 ? (long long)Arena::size<T>(2 * (size_t)hs.Cs.nrows) : 0);
+  const long long room = std::max(0LL, std::min(bound, ar.spared));
+  ar.spared -= room;
+  if (by_counts) {
+    ar.bytes += room;
+    ar.peak = std::max(ar.peak, ar.bytes);
     return;
   }
+  SolidPatchHost h;
+  if (!build_solid_patches(hs.Cs, ref_xy, pr.cs_k - 1, f64, NT, h) ||
+      4 * sizeof(T) * (size_t)h.max_loc > kClSmemCap)   // an outer layer too long for the iterate's two copies
+    return;
+  const size_t need = Arena::size<int>(h.poff.size()) + Arena::size<int>(h.cnt.size()) + Arena::size<int>(h.gid.size()) +
+                      Arena::size<int>(h.roff.size()) + Arena::size<T>(h.val.size()) +
+                      Arena::size<uint16_t>(h.col.size()) +
+                      (h.launches > 1 ? Arena::size<T>(2 * (size_t)hs.Cs.nrows) : 0);
+  if ((long long)need > room) return;
   SolidPatches<T>& d = pr.sc;
   d.np = h.np;
   d.steps = h.steps;
@@ -1238,6 +1253,13 @@ static void setup_solid_patches(Arena& ar, const HostSetup& hs, const double* re
     CK(cudaFuncSetAttribute(k_solid_cheb<T, kScWide, 1, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
     CK(cudaFuncSetAttribute(k_solid_cheb<T, kScWide, 2, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
   }
+}
+
+// The mass solves' matrices: patches, or C_s itself for the per-step launches.
+template <class T>
+static void setup_mass_solves(Problem& P, Prec<T>& pr, const double* ref_xy) {
+  setup_solid_patches<T>(P.ar, P.hs, ref_xy, P.by_counts, pr);
+  if (pr.sc.np == 0) pr.Cs = upload_sell<T>(P.ar, to_sell(P.hs.Cs));
 }
 
 template <class T>
@@ -2394,12 +2416,11 @@ static void build_hierarchies(Problem& P) {
 }
 
 template <class T>
-static void build_prec(Problem& P, Prec<T>& pr, const FullOp<T>& op, const double* ref_xy) {
+static void build_prec(Problem& P, Prec<T>& pr, const FullOp<T>& op) {
   Arena& ar = P.ar;
   alloc_mg<T>(ar, P.hs, pr.mgU, P.prm.autotune == 1, P.stream);
   alloc_mg<T>(ar, P.hs, pr.mgP, P.prm.autotune == 1, P.stream);
   pr.op = op;
-  pr.Cs = upload_sell<T>(ar, to_sell(P.hs.Cs));
   pr.As = upload_sell<T>(ar, to_sell(P.hs.As));
   if (P.prm.solid_law == 1) {
     pr.KT.nrows = P.nS; pr.KT.BR = 2; pr.KT.BC = 2; pr.KT.NV = 4; pr.KT.kron = false;
@@ -2415,7 +2436,6 @@ static void build_prec(Problem& P, Prec<T>& pr, const FullOp<T>& op, const doubl
   pr.sb = ar.alloc<T>(n2); pr.sx = ar.alloc<T>(n2); pr.sx2 = ar.alloc<T>(n2); pr.sd = ar.alloc<T>(n2);
   pr.cs_k = P.prm.cs_degree;
   pr.chs = cheb_coeffs(P.hs.cs_lo, P.hs.cs_hi, pr.cs_k);
-  setup_solid_patches<T>(ar, P.hs, ref_xy, pr);
   const size_t nf = 2 * (size_t)P.nU + 3 * (size_t)P.nP;
   pr.ru = ar.alloc<T>(2 * (size_t)P.nU);
   pr.t = ar.alloc<T>(nf);
@@ -2806,11 +2826,14 @@ static void allocate_problem(Problem& P, const double* ref_xy, const int* tris_h
   P.part = ar.alloc<double>((size_t)std::max(P.red_blocks, 64) * (m + 2));
   P.ctl = ar.alloc<Ctl>(1);
   P.op64 = make_op<double>(P, P.p64, P.cf_val, P.cft_val);
-  build_prec<double>(P, P.p64, P.op64, ref_xy);
+  build_prec<double>(P, P.p64, P.op64);
   if (P.prm.precision == 1) {
     P.op32 = make_op<float>(P, P.p32, P.cf_val32, P.cft_val32);
-    build_prec<float>(P, P.p32, P.op32, ref_xy);
+    build_prec<float>(P, P.p32, P.op32);
   }
+  // FP32 first: a mixed problem's solves take it
+  if (P.prm.precision == 1) setup_mass_solves<float>(P, P.p32, ref_xy);
+  setup_mass_solves<double>(P, P.p64, ref_xy);
   // The pairs of the exact rule live in the Krylov basis, idle while C_f is
   // assembled; where it is too short (few vectors, a body much finer than the grid)
   // they take memory spared elsewhere, or each row forms its own.
@@ -2886,13 +2909,15 @@ static void upload_state(Problem& P, const double* u, const double* X) {
   if (u || X) CK(cudaStreamSynchronize(P.stream));
 }
 
+// by_counts: the mesh stands for every mesh of its counts
 static size_t footprint_impl(const fsi_params& prm0, int n_nodes, int n_tris, const double* ref_xy,
-                             const int* tris) {
+                             const int* tris, bool by_counts) {
   fsi_params prm = with_defaults(prm0);
   check_params(prm, n_nodes, n_tris);
   Problem P;
   P.prm = prm;
   P.ar.count_only = true;
+  P.by_counts = by_counts;
   P.N = prm.N;
   VNum vn(prm.N);
   P.nU = vn.n; P.nP = prm.N * prm.N; P.nS = n_nodes; P.nTri = n_tris; P.nPts = elem_points(prm) * n_tris;
@@ -2941,7 +2966,7 @@ size_t fsi_footprint_bytes(const fsi_params* params, int n_solid_nodes, int n_tr
           const int j = t % (m - 1);
           tr[4 * t] = j; tr[4 * t + 1] = j + 1; tr[4 * t + 2] = m + j + 1; tr[4 * t + 3] = m + j;
         }
-        return footprint_impl(*params, n_solid_nodes, n_tris, xy.data(), tr.data());
+        return footprint_impl(*params, n_solid_nodes, n_tris, xy.data(), tr.data(), true);
       }
       // quadrilaterals (centre, three consecutive ring nodes): convex and
       // counter-clockwise while three ring steps span less than half a turn
@@ -2951,7 +2976,7 @@ size_t fsi_footprint_bytes(const fsi_params* params, int n_solid_nodes, int n_tr
         const int c = 1 + (b % (n_solid_nodes - 1));
         tr[4 * t] = 0; tr[4 * t + 1] = a; tr[4 * t + 2] = b; tr[4 * t + 3] = c;
       }
-      return footprint_impl(*params, n_solid_nodes, n_tris, xy.data(), tr.data());
+      return footprint_impl(*params, n_solid_nodes, n_tris, xy.data(), tr.data(), true);
     }
     if (n_solid_nodes < 5) {
       // too few ring nodes for a fan (its closing triangle would span half a
@@ -2974,14 +2999,14 @@ size_t fsi_footprint_bytes(const fsi_params* params, int n_solid_nodes, int n_tr
         if (c % 2 == 0) { tr[3 * t] = j; tr[3 * t + 1] = j + 1; tr[3 * t + 2] = m + j + 1; }
         else { tr[3 * t] = j; tr[3 * t + 1] = m + j + 1; tr[3 * t + 2] = m + j; }
       }
-      return footprint_impl(*params, n_solid_nodes, n_tris, xy.data(), tr.data());
+      return footprint_impl(*params, n_solid_nodes, n_tris, xy.data(), tr.data(), true);
     }
     for (int t = 0; t < n_tris; ++t) {
       const int a = 1 + t % (n_solid_nodes - 1);
       const int b = 1 + (a % (n_solid_nodes - 1));
       tr[3 * t] = 0; tr[3 * t + 1] = a; tr[3 * t + 2] = b;
     }
-    return footprint_impl(*params, n_solid_nodes, n_tris, xy.data(), tr.data());
+    return footprint_impl(*params, n_solid_nodes, n_tris, xy.data(), tr.data(), true);
   } catch (...) {
     return 0;
   }
@@ -2998,7 +3023,7 @@ int fsi_create_problem_budget(const fsi_params* params, const fsi_solid_mesh* me
     for (size_t i = 0; i < (size_t)elem_nodes(prm) * mesh->n_tris; ++i)
       if (mesh->tris[i] < 0 || mesh->tris[i] >= mesh->n_nodes) return FSI_ERR_INVALID;
     if (budget_bytes > 0) {
-      const size_t need = footprint_impl(prm, mesh->n_nodes, mesh->n_tris, mesh->ref_xy, mesh->tris);
+      const size_t need = footprint_impl(prm, mesh->n_nodes, mesh->n_tris, mesh->ref_xy, mesh->tris, false);
       if (need > budget_bytes) return FSI_ERR_BUDGET;
     }
     h = new fsi_problem();

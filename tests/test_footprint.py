@@ -23,6 +23,13 @@ PAIRS = [    # the exact rule's table of pairs
     (128, 50, dict(precision=1, restart=60, mg_fused=-1, coupling=1), 735133952, None),
     (16, 30, dict(precision=1, restart=60, coupling=1), 76600320, 73876072),
 ]
+SOLID = [    # the patches of the mass solves
+    (4, 30, dict(precision=1, restart=1, mg_fused=-1, mg_cluster=-1), 11008000, 9809207),
+    (2, 9, dict(precision=0, restart=1, solid_law=1, gamma=1.0, eta=1.0), 1151488, 1004318),
+    (24, 9, dict(precision=1, restart=60, mg_fused=-1), 36127488, 35069202),
+    (64, 9, dict(precision=1, restart=1, mg_fused=-1, mg_cluster=-1, solid_law=1, gamma=1.0, eta=1.0), 124329472, 117506489),
+    (6, 30, dict(precision=1, restart=60, coupling=1), 20155648, 18956814),
+]
 
 
 def _library():
@@ -49,7 +56,7 @@ def _admits(fsi, prm, xy, tris, budget):
         return e.code != fsi.FSI_ERR_BUDGET
 
 
-@pytest.mark.parametrize("N,rings,opt,counts,mesh", COARSE + PAIRS)
+@pytest.mark.parametrize("N,rings,opt,counts,mesh", COARSE + PAIRS + SOLID)
 def test_budgets_of_the_stored_form_still_admit(N, rings, opt, counts, mesh):
     fsi = _library()
     xy, tris = fi.ring_disk_mesh(rings, 0.2, (0.47, 0.52))
