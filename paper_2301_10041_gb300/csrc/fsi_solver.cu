@@ -1958,13 +1958,13 @@ __global__ void k_basis(int n2, double* __restrict__ V, size_t ld, const double*
 // refinement if needed, the Givens step, the next basis vector) with cluster
 // barriers between them.  As launches, the passes of a 7400-unknown problem take
 // 33 us, nearly all of it launch boundaries, last-block hand-overs and the
-// FP64 latency of their reductions; 16 SMs hold the FP64 work of up to 1024
-// rows each (kGsClusterRows) in about the time the hand-overs take.
+// FP64 latency of their reductions; 16 SMs hold the FP64 work of up to 512 rows
+// each (kGsClusterRows) in about the time the hand-overs take, in short cycles.
 // Rows are worked by four warps, one per SM quarter: an FP64 instruction holds
 // a quarter's pipe for 64 cycles, so more warps would only repeat the butterflies.
 constexpr int kGsCluster = 16;
 constexpr int kGsWorkers = 128;                       // threads that own row pairs
-constexpr int kGsPairs = 4;                           // row pairs of one of them, at most
+constexpr int kGsPairs = 2;                           // row pairs of one of them, at most
 constexpr int kGsClusterRows = 2 * kGsWorkers * kGsPairs;
 
 struct GsClusterShared {
@@ -2559,11 +2559,20 @@ static cudaLaunchConfig_t gs_cluster_config(cudaLaunchAttribute* at, cudaStream_
 }
 
 // Whether the problem's orthogonalisation runs as one cluster: its rows fit, and
-// the device schedules a cluster of this (non-portable) size.  At 16 384 unknowns
-// the cluster's FP64 work has grown to what the separate launches cost.
+// the device schedules a cluster of this (non-portable) size.  A row pair more per
+// worker makes each basis vector dearer (0.77, 1.22, 1.68 and 2.13 us a vector at
+// one to four pairs, 0.7 to 0.85 as separate launches), so the line lies where the
+// cycles of a precision still gain, in us an iteration with j vectors, cluster
+// against launches:
+//   FP64, cycles as long as the solve, one pair (n <= 4096): n = 3366 86 / 98 at
+//     j = 10, 96 / 99 at 24, 162 / 167 at 112, 248 / 259 at 220; but n = 5110
+//     104 / 110 at 10, 138 / 136 at 40, 230 / 206 at 112, 360 / 287 at 220;
+//   mixed, cycles of some 10 vectors (inner_rtol), two pairs (n <= 8192): n = 7014
+//     54.4 / 56.4 at 10, 70.7 / 68.9 at 24; but n = 16054 75 / 68 at 10, 143 / 88 at
+//     40, and FP64 n = 9726 103 / 104 at 10, 156 / 133 at 40.
 template <class T>
 static bool gs_cluster_fits(size_t n) {
-  if (n > (size_t)kGsCluster * kGsClusterRows) return false;
+  if (n > (size_t)kGsCluster * kGsClusterRows / (sizeof(T) == 8 ? 2 : 1)) return false;
   if (cudaFuncSetAttribute(k_gs_cluster<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
     cudaGetLastError();
     return false;
