@@ -455,7 +455,7 @@ def large_n_roofline(fsi, stream, device_index, peak, N):
                                    max_it=MAX_IT, stokes_its=STOKES_ITS, **arm_settings(0))
     prob64.assemble_step()
     ms, by = prob64.time_kernel(3, reps=30)
-    out["sell_velocity_chebyshev_f64"] = {"us": ms * 1e3, "bytes": by, "gbs": by / ms / 1e6,
+    out["velocity_chebyshev_f64"] = {"us": ms * 1e3, "bytes": by, "gbs": by / ms / 1e6,
                                           "frac": by / ms / 1e6 / peak}
     prob64.close()
     out["clocks"] = clocks.stop()

@@ -277,8 +277,9 @@ int fsi_graph_kernel_counts(const fsi_problem* p, int* counts);
  * stream with CUDA events, each launch after a 256 MiB write that evicts
  * L2, on the current data of the problem.  which: 0 full operator in FP32
  * (precision 1 only), 1 full operator in FP64 (residual form), 2 finest
- * velocity Chebyshev smoothing step in FP32 (precision 1 only), 3 the same in
- * FP64; 4 and 5 (precision 1 only): one whole V-cycle on the velocity /
+ * velocity Chebyshev smoothing step on the stored matrix in FP32 (precision 1
+ * only), 3 the same step in FP64 as the V-cycle runs it (matrix-free or
+ * stored); 4 and 5 (precision 1 only): one whole V-cycle on the velocity /
  * pressure-Laplacian hierarchy in FP32, with L2 left warm as inside a solve
  * (bytes: every level's vectors once, the stored matrices of the levels that
  * run the per-level kernels once per application, the dense coarsest inverse

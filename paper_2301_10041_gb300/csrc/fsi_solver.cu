@@ -3499,7 +3499,7 @@ int fsi_time_kernel(fsi_problem* h, int which, int reps, double* avg_ms, double*
     } held;
     Sell<float> A2;
     Sell<double> A3;
-    if (which == 2 || which == 3) {
+    if (which == 2 || (which == 3 && P.p64.mgU.lv[0].mfo.N == 0)) {
       const SellHost sa = to_sell(A0);
       if (which == 2) A2 = upload_sell<float>(held, sa);
       else A3 = upload_sell<double>(held, sa);
@@ -3528,12 +3528,13 @@ int fsi_time_kernel(fsi_problem* h, int which, int reps, double* avg_ms, double*
           *bytes = sell_bytes<float>(A0) + 6.0 * L.n * sizeof(float);
           break;
         }
-        case 3: {  // the same, FP64
+        case 3: {  // finest velocity Chebyshev step as the FP64 V-cycle runs it
           MGLevel<double>& L = P.p64.mgU.lv[0];
           SpmvArgs<double> a;
           a.x = L.x; a.y = L.x2; a.z = L.b; a.d = L.d; a.dinv = L.dinv; a.c1 = 0.5; a.c2 = 0.5;
-          sell_launch(A3, MODE_CHEB, a, s);
-          *bytes = sell_bytes<double>(A0) + 6.0 * L.n * sizeof(double);
+          if (L.mfo.N > 0) level_launch(L, MODE_CHEB, a, s);
+          else sell_launch(A3, MODE_CHEB, a, s);
+          *bytes = (L.mfo.N > 0 ? 0.0 : sell_bytes<double>(A0)) + 6.0 * L.n * sizeof(double);
           break;
         }
         case 4:    // one V-cycle on the Q2 velocity hierarchy, FP32

@@ -65,3 +65,16 @@ def test_fp32_richardson_residual_matches_the_stored_one(N):
     finally:
         on.close()
         off.close()
+
+
+@pytest.mark.parametrize("N,mg_fused,stored", [(16, 0, True), (32, 0, False), (64, 0, False), (64, -1, True)])
+def test_fp64_smoothing_step_is_timed_as_it_runs(N, mg_fused, stored):
+    """The timing hook's FP64 smoothing step: matrix-free from 32 cells (the six
+    vectors and nothing else), on the stored blocks below and with mg_fused = -1."""
+    from paper_2301_10041_gb300 import fsi
+    g = fsi.problem_from_case(_case(N), precision=0, restart=5, mg_fused=mg_fused)
+    try:
+        ms, by = g.time_kernel(3, 1)
+        assert ms > 0 and (by > 6 * 8 * g.n_u) == stored and by >= 6 * 8 * g.n_u
+    finally:
+        g.close()
