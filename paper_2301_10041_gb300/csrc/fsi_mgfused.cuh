@@ -91,11 +91,16 @@ constexpr int mf_pres_blk(int v, int y, int x) { return kMfPresVar * v + kMfPres
 // than one tile size for all levels.  Where there are enough tiles to fill the
 // chip, larger ones repeat less of their neighbours' work: velocity levels above
 // 128 cells take 16-node tiles (256 cells, down / residual down / up: 14.3 / 24.0 /
-// 12.5 -> 9.9 / 16.1 / 8.4 us; 160 cells 7.2 / 12.9 / 6.2 -> 6.5 / 9.9 / 5.1),
+// 12.5 -> 9.9 / 16.1 / 8.4 us; 160 cells 7.2 / 12.9 / 6.2 -> 6.5 / 9.9 / 5.1, at
+// degree 2; at every degree 1 to 4 they win although at 3 and 4 only one CTA fits on
+// an SM: the whole V-cycle, warm, 54 -> 51 and 71 -> 66 us on 160 cells, 78 -> 68
+// and 109 -> 89 on 256, 178 -> 149 and 268 -> 197 on 448),
 // pressure levels 8-cell tiles from 512 cells on (on 256 they are slower, 8.2 ->
-// 10.2 us).  Up to 32 cells a velocity level takes 4-node tiles: 64 CTAs of 384 threads instead of 16 of 512, down 3.35 -> 3.0 us,
-// up 3.3 -> 2.9 us on 32 cells (but 3.4 -> 5.8 us on 64, where they do not all fit
-// beside their four times repeated overlap).
+// 10.2 us).  Up to 32 cells a velocity level takes 4-node tiles: 64 CTAs of 384
+// threads instead of 16 of 512, down 3.35 -> 3.0 us, up 3.3 -> 2.9 us on 32 cells (but
+// 3.4 -> 5.8 us on 64, where they do not all fit beside their four times repeated
+// overlap).  By degree, cold, the whole V-cycle on 20 to 32 cells: equal at 1 to 3,
+// 19.3 -> 17.2 to 20.3 -> 18.4 us at 4.
 __host__ __device__ __forceinline__ int mf_tile_u(int N) { return N > 128 ? 16 : (N > 32 ? 8 : 4); }
 __host__ __device__ __forceinline__ int mf_tile_p(int N) { return N >= 512 ? 8 : 4; }
 // Threads of a velocity launch.  A launch's time on these grids is one CTA's
