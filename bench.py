@@ -365,9 +365,9 @@ def roofline(prob, args):
     FP32 FMA rate (algorithmic FLOPs without the overlap work of the tiles)
     and its HBM fraction is reported beside it.  Timed live on the library's
     stream with CUDA events, L2 evicted before every launch.  The other fused
-    launches, the FP32 full-system operator (sparse, HBM-bound) and the
-    per-level sparse smoothing step (the kernel of the FP64 arm and of
-    mg_fused = -1) are reported beside it."""
+    launches, the FP32 full-system operator (matrix-free fluid rows, latency-
+    bound at this size) and the smoothing step on the stored matrix (the kernel
+    of mg_fused = -1) are reported beside it."""
     peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))) if os.path.exists(
         os.path.join(ROOT, "MEASURED_PEAKS.json")) else {}
     peak = peaks.get("hbm_gbs", 6800.0)
@@ -417,7 +417,7 @@ def roofline(prob, args):
                 "achieved": d["gbs"], "peak": peak, "unit": "GB/s", "frac": d["hbm_frac"], "traffic": None,
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs" if peaks else "fallback 6800 GB/s",
                 "launch_us": d["us"], "algorithmic_bytes": d["bytes"], "others": out}
-    return {"bound": "alu", "kernel": "k_mfu_down<float,8,2,512> (fused down launch, finest velocity level)",
+    return {"bound": "alu", "kernel": "k_mfu_down<float,8,2,512,2> (fused down launch, finest velocity level)",
             "achieved": dom["tflops"], "peak": alu_peak, "unit": "TFLOP/s", "frac": dom["alu_frac"],
             "traffic": traffic, "peak_source": "derived: FP32 FMA lanes x 2 x max SM clock",
             "peak_derivation": alu_how, "launch_us": dom["us"], "algorithmic_flops": dom["flops"],

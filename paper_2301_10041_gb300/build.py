@@ -1,6 +1,6 @@
 """In-tree build of the CUDA library ``_lib/libfsi_gb300.so`` for sm_103a.
 
-The two translation units are compiled in parallel with nvcc and linked
+The three translation units are compiled in parallel with nvcc and linked
 with the static CUDA runtime; no cmake and no torch extension machinery.
 """
 from __future__ import annotations

@@ -50,8 +50,8 @@ struct CudaError : std::runtime_error {
 
 static inline unsigned nblk(size_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
-// Every kernel of the library (but the cluster V-cycle) is launched through
-// here.  The launches carry programmatic stream serialisation, so a kernel may
+// Every kernel of a step but the two cluster launches (the coarse levels of a
+// V-cycle, the orthogonalisation of a small problem) is launched through here.  The launches carry programmatic stream serialisation, so a kernel may
 // be scheduled while its predecessor on the stream finishes; each kernel
 // waits for its producers (griddepcontrol.wait, in pdl_begin() or the fused
 // kernels' wrapper) before it touches memory.  With the fused multigrid
@@ -1155,10 +1155,6 @@ struct Problem {
 };
 
 // ------------------------------------------------------- solid block A_22^-1
-// Exact up to the two C_s solves (Chebyshev-Jacobi on [1/2, 2], Wathen's
-// bounds for the Jacobi-scaled P1 mass matrix):
-//   X = -dt C_s^-1 r_l,   lambda = C_s^-1 (A_s X - r_X),
-// with r_l = v_l - C_f z_u for the block-triangular preconditioner.
 // One mass solve C_s x = b by its patches: cs_k Chebyshev-Jacobi steps (the
 // first one the start x = d = c0 D^-1 b) over sc_launches launches.  b is
 // scale bsrc, or K kx - bsrc when kx is given.
@@ -1262,6 +1258,10 @@ static void setup_mass_solves(Problem& P, Prec<T>& pr, const double* ref_xy) {
   if (pr.sc.np == 0) pr.Cs = upload_sell<T>(P.ar, to_sell(P.hs.Cs));
 }
 
+// Exact up to the two C_s solves (Chebyshev-Jacobi on [1/2, 2], Wathen's
+// bounds for the Jacobi-scaled P1 mass matrix):
+//   X = -dt C_s^-1 r_l,   lambda = C_s^-1 (A_s X - r_X),
+// with r_l = v_l - C_f z_u for the block-triangular preconditioner.
 template <class T>
 static void solid_launch(Problem& P, Prec<T>& pr, cudaStream_t s) {
   const int n2 = 2 * P.nS;
