@@ -628,7 +628,7 @@ static void plan_mg(const HostSetup& hs, bool pressure, int degree, MG<T>& mg, b
 // fused levels and in the cluster (their own images; a count without a device takes
 // the cluster for granted and so counts its levels here too), and not A where the
 // level's product is matrix-free.  With the level-0 rows of the operator, which
-// make_op leaves out likewise: 7.5 -> 4.4 GB on 512 cells in mixed precision with
+// make_op leaves out likewise: 7.6 -> 4.4 GB on 512 cells in mixed precision with
 // 60 basis vectors.
 template <class T>
 static void alloc_mg(Arena& ar, const HostSetup& hs, MG<T>& mg, bool tune, cudaStream_t s) {
