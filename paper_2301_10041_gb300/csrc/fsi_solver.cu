@@ -461,7 +461,7 @@ static void upload_classes(Arena& ar, MG<T>& mg, const SymMap& sym, const std::v
 // 11.7 -> 7.3 us, 768: 5.6 -> 4.9).  The full FP64 inverse stays on the device only
 // where a cluster launch reads it, and the classes go through the host one at a time,
 // so that nothing but one class stands beside it: a mixed problem of 16 cells and
-// 271 solid nodes takes 32 MB at most, 73 with the inverses kept beside the classes.
+// 271 solid nodes takes 33 MB at most, 73 with the inverses kept beside the classes.
 static void build_coarse(Arena& ar, const HostSetup& hs, bool pressure, MG<double>& m64, MG<float>* m32, int cl_max,
                          cudaStream_t s) {
   const int n = pressure ? hs.coarse_nL : hs.coarse_nA, ld = dense_ld<double>(n);
@@ -2387,8 +2387,9 @@ static fsi_params with_defaults(fsi_params p) {
   return p;
 }
 
-// The four hierarchies' plans and coarsest solves, before any other memory is
-// taken: the full inverses that the creation needs go back before the rest comes.
+// The four hierarchies' plans and coarsest solves, before the memory of the levels,
+// the operators and the basis is taken: the full inverses that the creation needs go
+// back before the rest comes.
 static void build_hierarchies(Problem& P) {
   const bool mixed = P.prm.precision == 1;
   // the FP64 levels are matrix-free products launch by launch (the FP32 ones
@@ -2748,7 +2749,6 @@ static void allocate_problem(Problem& P, const double* ref_xy, const int* tris_h
   Arena& ar = P.ar;
   const HostSetup& hs = P.hs;
   const int npe = elem_nodes(P.prm);
-  build_hierarchies(P);
   P.tris = ar.upload(std::vector<int>(tris_h, tris_h + npe * (size_t)P.nTri));
   P.area = ar.upload(npe == 4 ? hs.pt_w : hs.tri_area);
   P.ntp = ar.upload(hs.node_tri_ptr);
@@ -2822,6 +2822,7 @@ static void allocate_problem(Problem& P, const double* ref_xy, const int* tris_h
   P.lift_u = ar.upload(hs.lift_u);
   P.M64 = upload_sell<double>(ar, to_sell(hs.M));
   P.Cs64 = upload_sell<double>(ar, to_sell(hs.Cs));
+  build_hierarchies(P);
   const int m = P.m;
   P.V = ar.alloc<double>((size_t)(m + 1) * P.n);
   if (P.prm.precision == 1) P.Z = ar.alloc<float>((size_t)m * P.n);
